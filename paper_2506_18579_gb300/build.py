@@ -17,9 +17,9 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "librtgd.so")
-SOURCES = ["rtgd_api.cu", "rtgd_kernels.cu", "rtgd_noalloc.cu", "rtgd_server.cu", "rtgd_peaks.cu"]
-HEADERS = [os.path.join(INCLUDE, "rtgd.h"), os.path.join(CSRC, "rtgd_device.cuh"),
-           os.path.join(CSRC, "rtgd_internal.h")]
+SOURCES = ["rtgd_api.cu", "rtgd_kernels.cu", "rtgd_fp64.cu", "rtgd_noalloc.cu", "rtgd_server.cu", "rtgd_peaks.cu"]
+HEADERS = [os.path.join(INCLUDE, "rtgd.h")] + [os.path.join(CSRC, h) for h in (
+    "rtgd_device.cuh", "rtgd_fan.cuh", "rtgd_fp64.cuh", "rtgd_internal.h")]
 NVCC = os.environ.get("NVCC", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE, "-I" + CSRC]

@@ -222,6 +222,7 @@ rt_err make_plan(const rt_grid *grid, const rt_fan_desc *fan, size_t n_rays, con
     lp->threads = c.block_threads ? c.block_threads : 128;
     lp->blocks = 0;
     lp->lanes = 1;
+    if (fan->precision == RT_FP64) lp->fp64_rays = fp64_rays_per_warp((long long)n_rays, props(grid->device).sms);
     if (fan->precision == RT_MIXED) {
         int lanes = c.lanes_per_ray;
         if (lanes == 0) {

@@ -1,0 +1,759 @@
+// rtgd_fp64.cu -- the all-FP64 tracer.
+//
+// What bounds it: GB300 issues FP64 at 1/64 of the FP32 rate.  Measured: one
+// FP64 instruction occupies a warp for 64 cycles whether 1 or 32 of its lanes
+// are active and however many independent ones follow, and four or more warps
+// of an SM share a rate of one per 19 cycles.  So lanes are free and warp
+// instructions are not: with one ray per lane an evaluation took ~770 FP64
+// warp instructions (23.8 us) however few rays the warp still held.
+//
+// Layout: a block is one warp that holds up to eight rays.  While n of them
+// are in flight, each is carried by a group of G = 32 / 2^ceil(log2 n) lanes,
+// which share the evaluation's independent parts (the polynomials of the
+// weights, the 16 sample rows, the state components, the coordinates, the
+// divisions, the r/theta/phi components of the field and the ray equations):
+// ~250 FP64 instructions at G = 4, ~175 at G = 32 (7.7 us).  As rays end the
+// warp regroups, so that its last ray runs on all 32 lanes.  A ray's
+// arithmetic is the same operations in the same order for every G (only the
+// lane that performs them changes), so its record depends neither on G nor on
+// its warp mates.  Ray states live in shared memory (slots), so that
+// regrouping moves no data.  The host starts a warp with as many rays as fill
+// the GPU (fp64_rays_per_warp).  Measured, one thread per ray before / now:
+// 16 rays RK4 without a field 133 / 32 ms, one RKF45 ray 42.5 / 16.1 ms, 720
+// rays 189 / 69 ms, the 24,840-ray fan 418 / 174 ms.
+#include <cuda_runtime.h>
+#include <math.h>
+
+#include "rtgd_fan.cuh"
+#include "rtgd_fp64.cuh"
+
+namespace rtgd {
+
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+
+// Polynomials of the one-dimensional weights (Appendix A; Eq. 7 for
+// Catmull-Rom) as Horner coefficients, highest power first: kinds 0 and 1
+// are the weights of nodes j-1 and j, kinds 2 and 3 their derivatives.
+//   kind 0: t p4(t), kind 1: 1 + t^2 p3(t), kind 2: p4(t), kind 3: t p3(t)
+// with p4 of all five coefficients and p3 of the first four.
+__constant__ double c_poly[2][4][5] = {
+    {{1.0 / 6.0, -5.0 / 12.0, -1.0 / 6.0, 11.0 / 12.0, -0.5},
+     {-0.5, 1.25, 0.5, -2.25, 0.0},
+     {5.0 / 6.0, -5.0 / 3.0, -0.5, 11.0 / 6.0, -0.5},
+     {-2.5, 5.0, 1.5, -4.5, 0.0}},
+    {{0.0, 0.0, -0.5, 1.0, -0.5},
+     {0.0, 0.0, 1.5, -2.5, 0.0},
+     {0.0, 0.0, -1.5, 2.0, -0.5},
+     {0.0, 0.0, 4.5, -5.0, 0.0}}};
+
+// Shared memory of a block, in doubles.  Slot (one per ray): state, k1,
+// sin(theta) at the state, then the scalars below.
+enum {
+    kY = 0, kK1 = 6, kSth = 12, kP, kH, kHs, kApo, kRPrev, kDrPrev, kHPrev, kLa, kLfa, kLb, kLfb, kXfac, kAb0,
+    kInts,             // 4 doubles: 8 ints (kId ...)
+    kSlot = kInts + 5
+};
+enum { kId = 0, kMode, kSteps, kAtt, kEv, kFlags, kSide, kIt };
+enum { kK1Valid = 1, kHavePrev = 2, kLands = 4, kExits = 8 };
+// Scratch (one per group): derivatives k2..k6, stage state / new state, error
+// estimate, in-cell coordinates and cells of the three axes, the 24 weights,
+// the altitude, longitude and latitude sums.
+enum { cK = 0, cT = 30, cE = 36, cFrac = 42, cCell = 45 /* 3 ints */, cW = 47, cV = 71, cS = 103, cO = 115, cGroup = 119 };
+static_assert(kSlot % 2 == 1 && cGroup % 2 == 1, "odd strides spread the groups over the banks");
+constexpr int kMaxRays = 8;  // rays a warp starts with at most (G = 4)
+constexpr int kPoly = 4 * 5, kPow2 = 20;  // tables at the start of the shared memory
+
+// x / c for a constant c with rc = 1/c correctly rounded: one Newton
+// correction of x rc gives the correctly rounded quotient (Markstein's
+// theorem), 3 FP64 instructions instead of ~10.  Non-finite and tiny x take
+// the division.
+__device__ __forceinline__ double div_const(double x, double c, double rc) {
+    const double q = x * rc;
+    const double r = fma(-c, q, x);
+    const double d = fma(r, rc, q);
+    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+    return e - 128u < 1800u || (__double2hiint(x) & 0x7fffffff) == 0 ? d : x / c;
+}
+
+__device__ __forceinline__ bool finite64(double x) {
+    return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
+}
+
+// max of two numbers at least one of which is >= +0 (not NaN): the order of
+// such doubles is the order of their bits as signed integers.
+__device__ __forceinline__ double max_bits(double a, double b) {
+    return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+}
+
+// Stage s (1..5) of Fehlberg 4(5): y + h * (its combination of k1..ks), one
+// component.  The fused multiply-adds are spelt out, here and below, because
+// the branches otherwise decide which products the compiler fuses.
+__device__ __forceinline__ double rkf45_stage(int s, double y, double h, const double *k1, const double *k, int c) {
+    const double k1c = k1[c];
+    if (s == 1) return fma(h, k1c * 0.25, y);
+    const double k2c = k[c];
+    if (s == 2) return fma(h, fma(3.0 / 32.0, k1c, __dmul_rn(9.0 / 32.0, k2c)), y);
+    const double k3c = k[6 + c];
+    if (s == 3)
+        return fma(h, fma(7296.0 / 2197.0, k3c, fma(1932.0 / 2197.0, k1c, -__dmul_rn(7200.0 / 2197.0, k2c))), y);
+    const double k4c = k[12 + c];
+    if (s == 4)
+        return fma(h, fma(-845.0 / 4104.0, k4c,
+                          fma(3680.0 / 513.0, k3c, fma(439.0 / 216.0, k1c, -__dmul_rn(8.0, k2c)))), y);
+    const double k5c = k[18 + c];
+    return fma(h, fma(-11.0 / 40.0, k5c,
+                      fma(1859.0 / 4104.0, k4c,
+                          fma(-3544.0 / 2565.0, k3c, fma(-8.0 / 27.0, k1c, __dmul_rn(2.0, k2c))))), y);
+}
+
+// Fourth-order solution and local error estimate (5th - 4th order) of one
+// component, the latter as h sum((b5_i - b4_i) k_i) so that it keeps full
+// relative precision (y5 - y4 would cancel against r ~ 6371 km).
+__device__ __forceinline__ void rkf45_end(double y, double h, const double *k1, const double *k, int c, double &yn,
+                                          double &e) {
+    const double k1c = k1[c], k3c = k[6 + c], k4c = k[12 + c], k5c = k[18 + c], k6c = k[24 + c];
+    yn = __dadd_rn(y, __dmul_rn(h, __dadd_rn(fma(2197.0 / 4104.0, k4c,
+                                                 fma(25.0 / 216.0, k1c, __dmul_rn(1408.0 / 2565.0, k3c))),
+                                             -div_const(k5c, 5.0, 1.0 / 5.0))));
+    e = h * fma(2.0 / 55.0, k6c,
+                fma(1.0 / 5.0 - 9.0 / 50.0, k5c,
+                    fma(28561.0 / 56430.0 - 2197.0 / 4104.0, k4c,
+                        fma(16.0 / 135.0 - 25.0 / 216.0, k1c, __dmul_rn(6656.0 / 12825.0 - 1408.0 / 2565.0, k3c)))));
+}
+
+// Step-size factor: 0.9 err^(-1/5) limited to [0.2, 5], rounded down to a
+// power of 2^(1/4), so step sizes change through discrete decisions only and
+// round-off in err cannot feed back into the step sequence.  The exponent
+// floor(4 log2 of it) is taken from a float logarithm wherever that is not
+// within 1e-3 of an integer (its error is below 1e-5); only the rest pays for
+// the double pow and logarithm (~150 FP64 instructions).
+__device__ __forceinline__ double step_factor64(double err, const double *pow2q) {
+    if (err == 0.0) return pow2q[19];  // 5 rounds down to 2^(9/4)
+    const float e = (float)err;
+    if (e > 1e-30f && e < 1e30f) {
+        const float l = -0.608012374f - 0.8f * __log2f(e);  // 4 log2(0.9 err^-0.2)
+        const float fl = floorf(l), d = l - fl;
+        if (d > 1e-3f && d < 0.999f) {
+            const int k = (int)fl;
+            return pow2q[(k < -10 ? -10 : (k > 9 ? 9 : k)) + 10];
+        }
+    }
+    const double fac = fmin(5.0, fmax(0.2, 0.9 * pow(err, -0.2)));
+    return exp2(floor(4.0 * log2(fac)) * 0.25);
+}
+
+// Peak of the cubic Hermite fit of r(s), s in [0,1], through (r0, h d0) and
+// (r1, h d1) with d0 > 0 >= d1 (zero of p'(s) by bisection).
+__device__ __noinline__ double hermite_peak(double r0, double r1, double d0, double d1, double h) {
+    const double m0 = h * d0, m1 = h * d1;
+    const double A = 2.0 * (r0 - r1) + m0 + m1;
+    const double B = 3.0 * (r1 - r0) - 2.0 * m0 - m1;
+    double lo = 0.0, hi = 1.0;
+    for (int it = 0; it < 60; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        const double dp = m0 + 2.0 * B * mid + 3.0 * A * mid * mid;
+        if (dp > 0.0) lo = mid;
+        else hi = mid;
+    }
+    const double s = 0.5 * (lo + hi);
+    return r0 + m0 * s + B * s * s + A * s * s * s;
+}
+
+// Group path to the face of one axis that the ray reaches next at coordinate
+// x with rate v (coordinate per km), HUGE_VAL if there is none.  Faces are
+// where the C1 interpolant's second derivatives jump (the right-hand side is
+// only C0 there), the grid's outer faces included.  Adaptive steps end just
+// past such a face instead of straddling it.
+__device__ __forceinline__ double face_axis64(double x, double v, int n) {
+    const bool up = v > 0.0, down = v < 0.0;
+    double F = up ? floor(x) + 1.0 : ceil(x) - 1.0;
+    if (up && F < 0.0) F = 0.0;
+    if (!up && F > (double)(n - 1)) F = (double)(n - 1);
+    const bool ok = (up && F <= (double)(n - 1)) || (down && F >= 0.0);
+    const double d = (F - x) / v;
+    return ok ? d : HUGE_VAL;
+}
+
+// tail64 by a quad of lanes: lane j = 0, 1, 2 carries the r, theta, phi
+// component (lane 3 repeats lane 2), and the independent quotients and the
+// partials FX, FL, FT of Appleton-Hartree stand side by side in lanes 0-2.
+// The same operations in the same order as tail64 (a lane that has nothing to
+// do in a shared instruction multiplies by 1 or adds -0, which changes
+// nothing): ~110 FP64 instructions instead of ~175, without a field ~30
+// instead of ~45.  d and dk receive dy[j] and dy[3 + j]; dXj is s.dX[j].
+__device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const StageIn<double> &s, double dXj, int j,
+                                            double &d, double &dk) {
+    auto from = [](double v, int lane) { return __shfl_sync(kFull, v, lane, 4); };
+    const double kr = s.k[0], kt = s.k[1], kp = s.k[2], X = s.X;
+    const double kj = j == 0 ? kr : j == 1 ? kt : kp;
+    const double kk = fma(kp, kp, fma(kr, kr, __dmul_rn(kt, kt)));
+    const double rc = __drcp_rn(j == 0 ? s.r : j == 1 ? s.sth : kk);
+    const double ir = from(rc, 0), ist = from(rc, 1);
+    double H, K, G;
+    if (rp.iso) {
+        H = __dmul_rn(0.5, dXj);
+        K = kj;
+        G = __dadd_rn(-kk, -X);
+    } else {
+        const double ikk = from(rc, 2);
+        // m_j: (my S) sph + (mx S) cph + mz C, and my cph - mx sph
+        const double sj = j == 0 ? s.sth : j == 1 ? s.cth : 1.0;
+        const double px = __dmul_rn(rp.m[0], sj), py = __dmul_rn(rp.m[1], sj);
+        const double mj = fma(j == 0 ? rp.m[2] : j == 1 ? -rp.m[2] : 1.0, j == 0 ? s.cth : j == 1 ? s.sth : -0.0,
+                              fma(py, j < 2 ? s.sph : s.cph, __dmul_rn(px, j < 2 ? s.cph : -s.sph)));
+        const double q = __dmul_rn(rp.R_E, ir);
+        const double A = __dmul_rn(__dmul_rn(__dmul_rn(rp.ab0, q), q), q);
+        const double A2 = __dmul_rn(A, A);
+        const double Yj = __dmul_rn(__dmul_rn(j == 0 ? -2.0 : 1.0, A), mj);
+        const double mr = from(mj, 0), mt = from(mj, 1);
+        const double kY = fma(kp, from(Yj, 2), fma(kr, from(Yj, 0), __dmul_rn(kt, from(Yj, 1))));
+        const double YY = __dmul_rn(A2, fma(__dmul_rn(3.0, mr), mr, 1.0));
+        const double smp = __dmul_rn(s.sth, mj);  // lanes 2, 3
+        // gYY: (-6 YY) ir, ((6 A2) mr) mt, ((6 A2) mr) smp
+        const double gYY = __dmul_rn(__dmul_rn(__dmul_rn(j == 0 ? -6.0 : 6.0, j == 0 ? YY : A2), j == 0 ? ir : mr),
+                                     j == 0 ? 1.0 : j == 1 ? mt : smp);
+        // gkY: (-3 kY) ir, A ((-2 kr) mt - kt mr), A ((-2 kr) smp + (kt cth) mp - kp (sth mr + cth mt))
+        const double m2kr = __dmul_rn(-2.0, kr), ktc = __dmul_rn(kt, s.cth);
+        const double inner = fma(s.sth, mr, __dmul_rn(s.cth, mt));
+        double e = __dmul_rn(j == 0 ? -3.0 : j == 1 ? -kt : ktc, j == 0 ? kY : j == 1 ? mr : mj);
+        e = fma(j == 0 ? 1.0 : m2kr, j == 0 ? -0.0 : j == 1 ? mt : smp, e);
+        e = fma(j < 2 ? 1.0 : -kp, j < 2 ? -0.0 : inner, e);
+        const double gkY = __dmul_rn(j == 0 ? ir : A, e);
+        const double L = __dmul_rn(__dmul_rn(kY, kY), ikk);
+        double T = __dadd_rn(YY, -L);
+        if (T < 0.0) T = 0.0;
+        const double u = __dadd_rn(1.0, -X);
+        const double L4u = __dmul_rn(__dmul_rn(4.0, L), u), L4uu = __dmul_rn(L4u, u);
+        const double S = sqrt(fma(T, T, L4uu));
+        // FX, FL, FT in lanes 0, 1, 2.  Groups of one warp may carry rays of both
+        // modes: the branches hold no shuffle (a warp-wide shuffle in a divergent
+        // branch would wait for lanes that never come).
+        const bool ord = rp.mode > 0;
+        const double u2 = __dmul_rn(2.0, u);
+        double W = 0.0, V = 0.0, D = 0.0, den;
+        if (ord) {
+            W = __dadd_rn(S, T);
+            V = __dadd_rn(W, __dmul_rn(__dmul_rn(2.0, L), u));
+            den = __dmul_rn(__dmul_rn(S, W), V);
+        } else {
+            D = __dadd_rn(fma(2.0, u, -T), -S);
+            den = __dmul_rn(S, D);
+        }
+        const double m = __drcp_rn(den);
+        // ordinary: iS = (W V) m, iW = (S V) m, 1/(1 + g) = ((S W) W) m; extraordinary: iS = D m, iD = S m
+        double iv = ord ? (j == 0 ? W : S) : (j == 0 ? D : S);
+        if (ord) {
+            if (j == 2) iv = __dmul_rn(S, W);
+            iv = __dmul_rn(iv, j < 2 ? V : W);
+        }
+        iv = __dmul_rn(iv, m);
+        const double iS = from(iv, 0), i1 = from(iv, 1), iopg = from(iv, 2);
+        double F;
+        if (ord) {
+            const double L2 = __dmul_rn(2.0, L), gg = __dmul_rn(__dmul_rn(L2, u), i1), opg = __dadd_rn(1.0, gg);
+            // gX = ((L2 (L4uu iS - W)) iW) iW, gL = u2 iW - (((L4uu u) iS) iW) iW, gT = -gg iS
+            double t = fma(j < 2 ? L4uu : -gg, j == 1 ? u : iS, j == 0 ? -W : -0.0);
+            t = __dmul_rn(t, j == 0 ? L2 : j == 1 ? iS : 1.0);
+            t = __dmul_rn(t, j < 2 ? i1 : 1.0);
+            t = __dmul_rn(t, j < 2 ? i1 : 1.0);
+            t = fma(j == 1 ? u2 : 1.0, j == 1 ? i1 : t, j == 1 ? -t : -0.0);
+            F = __dmul_rn(fma(X, t, j == 0 ? -opg : -0.0), __dmul_rn(iopg, iopg));
+        } else {
+            const double N = __dmul_rn(__dmul_rn(2.0, X), u), cD = __dmul_rn(fma(-4.0, X, 2.0), D);
+            const double t = fma(j == 0 ? L4u : j == 1 ? -__dmul_rn(u2, u) : -T, iS, j == 0 ? -2.0 : j == 1 ? -0.0 : -1.0);
+            F = __dmul_rn(fma(N, t, j == 0 ? -cD : -0.0), __dmul_rn(i1, i1));
+        }
+        const double FX = from(F, 0), FL = from(F, 1), FT = from(F, 2);
+        const double kYn = __dmul_rn(kY, ikk);
+        const double cL = __dmul_rn(__dadd_rn(FL, -FT), __dmul_rn(__dmul_rn(2.0, kY), ikk));
+        const double hf = __dmul_rn(0.5, cL);
+        H = __dmul_rn(-0.5, fma(cL, gkY, fma(FX, dXj, __dmul_rn(FT, gYY))));
+        K = fma(-hf, fma(-kYn, kj, Yj), kj);
+        G = fma(T, FT, fma(L, FL, fma(X, FX, -kk)));
+    }
+    const double iG = __drcp_rn(G), irs = __dmul_rn(ir, ist);
+    const double sc = j == 0 ? 1.0 : j == 1 ? ir : irs;
+    d = __dmul_rn(__dmul_rn(-K, iG), sc);
+    const double dr = from(d, 0), dt = from(d, 1), dp = from(d, 2);
+    // kp sth in lane 0, (kp r) cth in lanes 1, 2
+    const double kv = __dmul_rn(__dmul_rn(kp, j == 0 ? s.sth : s.r), j == 0 ? 1.0 : s.cth);
+    const double kps = from(kv, 0);
+    double t = __dmul_rn(j == 0 ? kt : j == 1 ? -kt : -kps, j == 0 ? dt : dr);
+    t = fma(j < 2 ? kv : -kv, j < 2 ? dp : dt, fma(H, iG, t));
+    dk = __dmul_rn(t, sc);
+}
+
+// dy/dP' at the stage state yt by the G lanes of a group (lane q, scratch C),
+// into out (6 doubles of shared memory) if write is set; coef: the weight
+// polynomials of the grid's interpolant; returns sin(theta).  Called by whole
+// warps only (it holds barriers and shuffles).
+template <int G>
+__device__ __forceinline__ double stage64(const GridDev &g, const RayPhys<double> &rp, const double yt[6], double *C,
+                                          const double *coef, int q, double *out, bool write) {
+    static_assert(G >= 4, "an axis and a component per lane of a quad");
+    StageIn<double> s;
+    s.r = yt[0];
+    s.k[0] = yt[3];
+    s.k[1] = yt[4];
+    s.k[2] = yt[5];
+    // cells: an axis per lane
+    int *cell = (int *)(C + cCell);
+    if (q < 3) {
+        int i;
+        double t;
+        const bool ok = cell64(grid_coord64(g, q, yt[0], yt[1], yt[2]), q == 0 ? g.n_lat : q == 1 ? g.n_lon : g.n_alt, i, t);
+        C[cFrac + q] = t;
+        cell[q] = ok ? i : -1;
+    }
+    // sines and cosines: theta on the even lanes, phi on the odd ones
+    double sn, cs;
+    sincos((q & 1) ? yt[2] : yt[1], &sn, &cs);
+    const double so = __shfl_xor_sync(kFull, sn, 1), co = __shfl_xor_sync(kFull, cs, 1);
+    s.sth = (q & 1) ? so : sn;
+    s.cth = (q & 1) ? co : cs;
+    s.sph = (q & 1) ? sn : so;
+    s.cph = (q & 1) ? cs : co;
+    __syncwarp();
+    const int ca = cell[0], cb = cell[1], cc = cell[2];
+    const bool inside = (ca | cb | cc) >= 0;
+    const int j = (q & 3) == 3 ? 2 : (q & 3);  // the component this lane carries
+    double dXj = 0.0;
+    s.X = 0.0;
+    if (__any_sync(kFull, inside)) {
+        // the 24 weights: weight p = 8 axis + 4 derivative + node, one polynomial each
+        for (int p = q; p < 24; p += G) {
+            const int node = p & 3, der = (p >> 2) & 1;
+            const bool right = node >= 2;
+            const bool outer = node == 0 || node == 3;  // nodes j-1, j+2
+            const double *cf = coef + (der * 2 + (outer ? 0 : 1)) * 5;
+            double t = C[cFrac + (p >> 3)];
+            t = right ? 1.0 - t : t;
+            double w = fma(t, cf[0], cf[1]);
+            w = fma(t, w, cf[2]);
+            w = fma(t, w, cf[3]);
+            // kinds 0, 2: one more Horner step; kind 1: t^2; kind 3: times t (adding -0 changes nothing)
+            const double w4 = fma(t, (der | (int)outer) ? w : t, outer ? cf[4] : -0.0);
+            const double w5 = __dmul_rn(w4, outer ? t : w);
+            w = der ? w4 : __dadd_rn(outer ? -0.0 : 1.0, w5);
+            C[cW + p] = (der && right) ? -w : w;
+        }
+        __syncwarp();
+        const long long sj = g.p_alt, si = (long long)g.p_lon * g.p_alt;
+        const double *base = g.pad64 + (long long)(inside ? ca : 0) * si + (long long)(inside ? cb : 0) * sj +
+                             (inside ? cc : 0);
+        // altitude rows (Eq. 13): row 4 a + b; with 32 lanes the upper half forms the derivative sums
+        if (G == 32) {
+            const int row = q & 15;
+            const double *p = base + (row >> 2) * si + (row & 3) * sj;
+            const double *w = C + cW + 16 + ((q >> 4) << 2);
+            C[cV + q] = fma(__ldg(p + 3), w[3], fma(__ldg(p + 2), w[2], fma(__ldg(p), w[0], __dmul_rn(__ldg(p + 1), w[1]))));
+        } else {
+            for (int row = q; row < 16; row += G) {
+                const double *p = base + (row >> 2) * si + (row & 3) * sj;
+                double v, dv;
+                row4<double>(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3), C + cW + 16, C + cW + 20, v, dv);
+                C[cV + row] = v;
+                C[cV + 16 + row] = dv;
+            }
+        }
+        __syncwarp();
+        // longitude: for each a the sums of v wb, v db, dv wb
+        for (int id = q; id < 12; id += G) {
+            const int a = id / 3, j = id - 3 * a;
+            const double *v = C + cV + (j == 2 ? 16 : 0) + 4 * a;
+            const double *w = C + cW + 8 + (j == 1 ? 4 : 0);
+            double sum = 0.0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) sum += v[b] * w[b];
+            C[cS + id] = sum;
+        }
+        __syncwarp();
+        // latitude, then to X and its derivatives along r, theta, phi: lane o
+        // forms X (0), dX/dtheta (1), dX/dphi (2), dX/dr (3)
+        for (int o = q; o < 4; o += G) {
+            const double *v = C + cS + (o == 3 ? 2 : o == 2 ? 1 : 0);
+            const double *w = C + cW + (o == 1 ? 4 : 0);
+            double sum = 0.0;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) sum += v[3 * a] * w[a];
+            const double c1 = o == 0 ? 1.0 : o == 1 ? g.inv_dlat : o == 2 ? g.inv_dlon : g.inv_dalt;
+            const double c2 = o == 1 || o == 2 ? kRad2Deg : 1.0;
+            C[cO + o] = (o == 1 ? -rp.xfac : rp.xfac) * sum * c1 * c2;
+        }
+        __syncwarp();
+        if (inside) {
+            s.X = C[cO];
+            dXj = C[cO + (j == 0 ? 3 : j)];
+        }
+    }
+    double d, dk;
+    tail64_quad(rp, s, dXj, j, d, dk);
+    if (write && q < 3) {
+        out[q] = d;
+        out[3 + q] = dk;
+    }
+    return s.sth;
+}
+
+// Raw final state of a ray into its record (the angles stand in the
+// ground-range and azimuth fields; finish_records_kernel turns them into the
+// outputs).
+__device__ __forceinline__ void write_raw(rt_ray_result *out, int id, double P, double th, double ph, double apo,
+                                          int status, int steps, int att, int ev) {
+    rt_ray_result r;
+    r.group_path_km = P;
+    r.ground_range_km = th;
+    r.az_dev_deg = ph;
+    r.apogee_km = apo;
+    r.land_lat_deg = 0.0;
+    r.land_lon_deg = 0.0;
+    r.status = status;
+    r.n_steps = steps;
+    r.n_attempts = att;
+    r.n_evals = ev;
+    out[id] = r;
+}
+
+// Runs the warp's rays, G lanes each, until at most half of the groups are
+// still in use; then packs the remaining rays' slots to the front of map.
+// One iteration is one step attempt (or one trial of the landing / exit
+// solve) of every ray.  Groups without a ray follow group 0's ray and write
+// nothing, so that the warp's barriers stay uniform.  The loop ends: every
+// iteration adds an attempt to each ray, and a ray takes at most max_steps of
+// them plus 60 trials.
+template <int G>
+__device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, double *slots, double *scratch,
+                                         const double *coef, const double *pow2q, int *map, int &n_act,
+                                         rt_ray_result *__restrict__ out) {
+    const int lane = threadIdx.x, grp = lane / G, q = lane % G;
+    const bool has = grp < n_act;
+    const int slot = map[has ? grp : 0];
+    double *S = slots + slot * kSlot;
+    int *SI = (int *)(S + kInts);
+    double *C = scratch + grp * cGroup;
+    const bool adaptive = f.integrator == RT_RKF45;
+    const int ns = adaptive ? 6 : 4;
+    const double RE = g.R_E;
+    RayPhys<double> rp;
+    rp.xfac = S[kXfac];
+    rp.ab0 = S[kAb0];
+    rp.R_E = RE;
+    rp.m[0] = g.m[0];
+    rp.m[1] = g.m[1];
+    rp.m[2] = g.m[2];
+    rp.iso = g.iso != 0;
+    rp.mode = SI[kMode];
+    double P = S[kP], h = S[kH], hs = S[kHs], apo = S[kApo], r_prev = S[kRPrev], dr_prev = S[kDrPrev], h_prev = S[kHPrev];
+    double la = S[kLa], lfa = S[kLfa], lb = S[kLb], lfb = S[kLfb];
+    int steps = SI[kSteps], att = SI[kAtt], ev = SI[kEv], flags = SI[kFlags], side = SI[kSide], it = SI[kIt];
+    const int id = SI[kId];
+    bool live = has;
+    const bool writer = q == 0;
+    __syncwarp();
+    for (;;) {
+        const unsigned am = __ballot_sync(kFull, live && writer);
+        const int n = __popc(am);
+        if (n == 0 || (G < 32 && 2 * n * G <= 32)) {
+            if (live && writer) {
+                S[kP] = P; S[kH] = h; S[kHs] = hs; S[kApo] = apo; S[kRPrev] = r_prev; S[kDrPrev] = dr_prev;
+                S[kHPrev] = h_prev; S[kLa] = la; S[kLfa] = lfa; S[kLb] = lb; S[kLfb] = lfb;
+                SI[kSteps] = steps; SI[kAtt] = att; SI[kEv] = ev; SI[kFlags] = flags; SI[kSide] = side; SI[kIt] = it;
+                map[__popc(am & ((1u << lane) - 1u))] = slot;
+            }
+            n_act = n;
+            __syncwarp();
+            return;
+        }
+        if (!live) {  // a group without a ray repeats plain steps from a fixed state
+            flags = kK1Valid;
+            h = f.h0;
+        }
+        const bool solving = (flags & (kLands | kExits)) != 0;
+        if (live && !solving && att >= f.max_steps) {
+            if (writer) write_raw(out, id, P, S[kY + 1], S[kY + 2], apo, RT_RAY_MAX_STEPS, steps, att, ev);
+            live = false;
+        }
+        double yt[6];
+        // k1 where it is not known (a new state)
+        const bool need = live && !(flags & kK1Valid);
+        if (__any_sync(kFull, need)) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) yt[i] = S[kY + i];
+            const double sth = stage64<G>(g, rp, yt, C, coef, q, S + kK1, need);
+            if (need) {
+                ++ev;
+                flags |= kK1Valid;
+                if (writer) S[kSth] = sth;
+            }
+            __syncwarp();
+        }
+        bool at_face = false;
+        if (!solving) hs = h;
+        if (adaptive) {
+            // distance to the next cell face, predicted linearly from k1; lateral
+            // faces count only inside the altitude span
+            const double y0 = S[kY], y1 = S[kY + 1], y2 = S[kY + 2];
+            const int ax = (q & 3) == 3 ? 2 : (q & 3);  // an axis per lane
+            const double x = grid_coord64(g, ax, y0, y1, y2);
+            const double v = (ax == 0 ? -S[kK1 + 1] : ax == 1 ? S[kK1 + 2] : S[kK1]) * (ax == 2 ? 1.0 : kRad2Deg) *
+                             (ax == 0 ? g.inv_dlat : ax == 1 ? g.inv_dlon : g.inv_dalt);
+            const double xc = __shfl_sync(kFull, x, 2, 4);
+            const bool in_alt = xc >= 0.0 && xc <= (double)(g.n_alt - 1);
+            double best = face_axis64(x, v, ax == 0 ? g.n_lat : ax == 1 ? g.n_lon : g.n_alt);
+            if (ax < 2 && !in_alt) best = HUGE_VAL;
+            best = fmin(best, __shfl_xor_sync(kFull, best, 1));
+            best = fmin(best, __shfl_xor_sync(kFull, best, 2));
+            if (!solving && best > 1e-3 * hs && best < hs) {
+                hs = best * (1.0 + 1e-4);
+                at_face = true;
+            }
+        }
+        const double k10 = S[kK1];
+        if (!solving) {
+            if (f.max_path > 0.0 && P + hs > f.max_path) hs = f.max_path - P;
+            if ((flags & kHavePrev) && dr_prev > 0.0 && k10 <= 0.0)
+                apo = fmax(apo, hermite_peak(r_prev, S[kY], dr_prev, k10, h_prev) - RE);
+            flags &= ~kHavePrev;
+        }
+        // the attempt: stages 1 .. ns-1, then the new state (and error estimate)
+#pragma unroll 1
+        for (int s = 1; s < ns; ++s) {
+#pragma unroll 1
+            for (int c = q; c < 6; c += G) {
+                const double y = S[kY + c];
+                C[cT + c] = adaptive ? rkf45_stage(s, y, hs, S + kK1, C + cK, c)
+                                     : fma(s == 3 ? hs : 0.5 * hs, s == 1 ? S[kK1 + c] : C[cK + 6 * (s - 2) + c], y);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 6; ++i) yt[i] = C[cT + i];
+            stage64<G>(g, rp, yt, C, coef, q, C + cK + 6 * (s - 1), true);
+            __syncwarp();
+        }
+        if (adaptive) {
+#pragma unroll 1
+            for (int c = q; c < 6; c += G) rkf45_end(S[kY + c], hs, S + kK1, C + cK, c, C[cT + c], C[cE + c]);
+        } else {
+            const double h6 = div_const(hs, 6.0, 1.0 / 6.0);
+#pragma unroll 1
+            for (int c = q; c < 6; c += G)
+                C[cT + c] = __dadd_rn(S[kY + c], __dmul_rn(h6, __dadd_rn(fma(2.0, C[cK + 6 + c], fma(2.0, C[cK + c], S[kK1 + c])),
+                                                                         C[cK + 12 + c])));
+        }
+        __syncwarp();
+        double yn[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) yn[i] = C[cT + i];
+        ++att;
+        ev += adaptive ? 5 : 3;
+        // error norm (<= 1 accepts), as documented in rtgd.h: the two quotients on the even and odd lanes
+        double fac = 1.0;
+        bool accept = true;
+        if (adaptive) {
+            const double r = S[kY], sth = S[kSth], ky = S[kY + 3], kt = S[kY + 4], kp = S[kY + 5];
+            const double e0 = C[cE], e1 = C[cE + 1], e2 = C[cE + 2], e3 = C[cE + 3], e4 = C[cE + 4], e5 = C[cE + 5];
+            const double kmag = sqrt(ky * ky + kt * kt + kp * kp);
+            double pos, kerr;
+            if (finite64(e0) && finite64(e1) && finite64(e2) && finite64(e3) && finite64(e4) && finite64(e5)) {
+                pos = max_bits(fabs(e0), max_bits(r * fabs(e1), r * sth * fabs(e2)));
+                kerr = max_bits(fabs(e3), max_bits(fabs(e4), fabs(e5)));
+            } else {
+                pos = fmax(fabs(e0), fmax(r * fabs(e1), r * sth * fabs(e2)));
+                kerr = fmax(fabs(e3), fmax(fabs(e4), fabs(e5)));
+            }
+            const double dp = f.atol + f.rtol * r, dk = f.rtol * fmax(kmag, 1e-3);
+            const double v = ((q & 1) ? kerr : pos) / ((q & 1) ? dk : dp);
+            const double err = fmax(v, __shfl_xor_sync(kFull, v, 1));
+            fac = step_factor64(err, pow2q);
+            accept = err <= 1.0;
+        }
+        // new state inside the grid's lat/lon span?  (an axis per lane)
+        int cell_i;
+        double cell_t;
+        const bool in_ax = cell64(grid_coord64(g, q & 1, yn[0], yn[1], yn[2]), (q & 1) ? g.n_lon : g.n_lat, cell_i, cell_t);
+        const bool lateral = __shfl_xor_sync(kFull, (int)in_ax, 1) && in_ax;
+        const double y0 = S[kY];
+        if (solving) {
+            // ground return or exit through the grid top: r(step(h*)) = R_E (or
+            // R_E + top) for h* in (0, step], Illinois regula falsi; sg makes the
+            // bracket function positive at the step start
+            const bool lands = (flags & kLands) != 0;
+            const double rt = lands ? RE : RE + g.top, sg = lands ? 1.0 : -1.0;
+            const double fc = sg * (yn[0] - rt);
+            ++it;
+            if (fabs(fc) < 1e-9 || it >= 60) {
+                P += hs;
+                ++steps;
+                if (!lands) apo = fmax(apo, yn[0] - RE);
+                if (live && writer)
+                    write_raw(out, id, P, yn[1], yn[2], apo, lands ? RT_RAY_LANDED : RT_RAY_ESCAPED, steps, att, ev);
+                live = false;
+            } else {
+                if (fc < 0.0) {
+                    lb = hs;
+                    lfb = fc;
+                    if (side == -1) lfa *= 0.5;
+                    side = -1;
+                } else {
+                    la = hs;
+                    lfa = fc;
+                    if (side == 1) lfb *= 0.5;
+                    side = 1;
+                }
+                hs = lb - lfb * (lb - la) / (lfb - lfa);
+            }
+        } else if (!accept) {
+            // the nominal step changes only by quantised factors of itself
+            h = h * fac;
+            if (h < f.hmin) {
+                if (live && writer)
+                    write_raw(out, id, P, S[kY + 1], S[kY + 2], apo, RT_RAY_STEP_UNDERFLOW, steps, att, ev);
+                live = false;
+            }
+        } else if (!(finite64(yn[0]) && finite64(yn[1]) && finite64(yn[2]) && finite64(yn[3]) && finite64(yn[4]) &&
+                     finite64(yn[5]))) {
+            if (live && writer) write_raw(out, id, P, S[kY + 1], S[kY + 2], apo, RT_RAY_NONFINITE, steps, att, ev);
+            live = false;
+        } else {
+            const bool lands = yn[0] < RE;
+            const bool exits = !lands && yn[0] - RE > g.top;
+            if (lands || exits) {
+                const double rt = lands ? RE : RE + g.top, sg = lands ? 1.0 : -1.0;
+                flags |= lands ? kLands : kExits;
+                la = 0.0;
+                lfa = sg * (y0 - rt);
+                lb = hs;
+                lfb = sg * (yn[0] - rt);
+                side = 0;
+                it = 0;
+                hs = lb - lfb * (lb - la) / (lfb - lfa);
+            } else {
+                P += hs;
+                ++steps;
+                apo = fmax(apo, yn[0] - RE);
+                flags = (flags | kHavePrev) & ~kK1Valid;
+                r_prev = y0;
+                dr_prev = k10;
+                h_prev = hs;
+                int status = RT_RAY_NOT_RUN;
+                if (yn[0] - RE >= g.alt0 && !lateral) status = RT_RAY_LEFT_GRID;
+                else if (f.max_path > 0.0 && P >= f.max_path - 1e-12) status = RT_RAY_MAX_PATH;
+                if (status != RT_RAY_NOT_RUN) {
+                    if (live && writer) write_raw(out, id, P, yn[1], yn[2], apo, status, steps, att, ev);
+                    live = false;
+                }
+                if (adaptive) h = fmin(fmax(h * (at_face ? fmin(1.0, fac) : fac), f.hmin), f.hmax);
+            }
+        }
+        // (a reader of the old state above has passed the barrier before the new one is written)
+        const bool moved = !(flags & kK1Valid);
+        __syncwarp();
+        if (live && writer && moved) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) S[kY + i] = yn[i];
+        }
+        __syncwarp();
+    }
+}
+
+// Bytes of shared memory of a block that starts with R rays.
+constexpr size_t fp64_smem_bytes(int R) {
+    return sizeof(double) * (size_t)(kPoly + kPow2 + R * (kSlot + cGroup)) + kMaxRays * sizeof(int);
+}
+static_assert(fp64_smem_bytes(kMaxRays) <= 48 * 1024, "fits the default shared-memory limit");
+
+// One warp per block; R rays (a power of two, at most kMaxRays) per warp at
+// the start.
+__global__ void __launch_bounds__(32) trace_fp64_kernel(const __grid_constant__ GridDev g,
+                                                        const __grid_constant__ FanDev f, int R,
+                                                        rt_ray_result *__restrict__ out) {
+    extern __shared__ double sm[];
+    double *coef = sm, *pow2q = coef + kPoly, *slots = pow2q + kPow2, *scratch = slots + R * kSlot;
+    int *map = (int *)(scratch + R * cGroup);
+    const int lane = threadIdx.x;
+    if (lane < kPoly) coef[lane] = (&c_poly[g.interp == 1 ? 1 : 0][0][0])[lane];
+    if (lane < kPow2) pow2q[lane] = exp2((double)(lane - 10) * 0.25);
+    // launch: |k| = mu at the transmitter (one ray per lane; spare lanes do nothing)
+    const long long claim = (long long)blockIdx.x * R + lane;
+    bool live = lane < R && claim < f.n_rays;
+    if (live) {
+        const long long ray = claim_to_ray(f, claim);
+        const RayParams p = ray_params(f, ray);
+        const RayPhys<double> rp = make_phys<double>(g, p.f_hz, p.mode);
+        double y[6], dummy[6], mu2 = 0.0;
+        launch_dir(f, p, y);
+        rhs64(g, rp, y, dummy, &mu2);
+        if (!(mu2 > 0.0)) {
+            write_raw(out, (int)ray, 0.0, y[1], y[2], f.tx_r - g.R_E, RT_RAY_NONFINITE, 0, 0, 1);
+            live = false;
+        } else {
+            const double mu = sqrt(mu2);
+            y[3] *= mu;
+            y[4] *= mu;
+            y[5] *= mu;
+            double *S = slots + lane * kSlot;
+            int *SI = (int *)(S + kInts);
+            for (int i = 0; i < 6; ++i) {
+                S[kY + i] = y[i];
+                S[kK1 + i] = 0.0;
+            }
+            S[kSth] = S[kP] = S[kRPrev] = S[kDrPrev] = S[kHPrev] = S[kLa] = S[kLfa] = S[kLb] = S[kLfb] = 0.0;
+            S[kH] = S[kHs] = f.h0;
+            S[kApo] = y[0] - g.R_E;
+            S[kXfac] = rp.xfac;
+            S[kAb0] = rp.ab0;
+            SI[kId] = (int)ray;
+            SI[kMode] = p.mode;
+            SI[kSteps] = SI[kAtt] = SI[kFlags] = SI[kSide] = SI[kIt] = 0;
+            SI[kEv] = 1;
+        }
+    }
+    const unsigned am = __ballot_sync(kFull, live);
+    if (live) map[__popc(am & ((1u << lane) - 1u))] = lane;
+    __syncwarp();
+    int n_act = __popc(am);
+    while (n_act > 0) {
+        if (n_act > 4) run_rays<4>(g, f, slots, scratch, coef, pow2q, map, n_act, out);
+        else if (n_act > 2) run_rays<8>(g, f, slots, scratch, coef, pow2q, map, n_act, out);
+        else if (n_act > 1) run_rays<16>(g, f, slots, scratch, coef, pow2q, map, n_act, out);
+        else run_rays<32>(g, f, slots, scratch, coef, pow2q, map, n_act, out);
+    }
+}
+
+}  // namespace
+
+// Rays a warp starts with.  An FP64 instruction takes a warp 64 cycles while
+// its SM holds fewer than ~3.4 warps and 19 cycles per resident warp above
+// that; kCost is what an evaluation takes in FP64 instructions at 4, 8, 16 and
+// 32 lanes per ray.  The size with the least product is taken.  Measured at 8 /
+// 4 / 2 / 1 rays per warp: 16 rays 54 / 43 / 36 / 32 ms, 522 rays 27 / 23 / 21 /
+// 19 ms, 3,232 rays 49 / 46 / 70 / 99 ms, 4,968 rays 135 / 142 / 146 / 173 ms,
+// 24,840 rays 174 / 223 / 352 ms / -.  More rays per warp (one or two lanes
+// each) were no faster at any size: 24,840 rays 184 ms with 32, 177 with 16.
+int fp64_rays_per_warp(long long n_rays, int sms) {
+    static const double kCost[4] = {226, 205, 190, 175};
+    double best = 1e300;
+    int R = 1;
+    for (int i = 0; i < 4; ++i) {
+        const int r = kMaxRays >> i;
+        const double warps = (double)((n_rays + r - 1) / r) / sms;
+        const double t = kCost[i] * (warps > 64.0 / 19.0 ? 19.0 * warps : 64.0);
+        if (t < best) {
+            best = t;
+            R = r;
+        }
+    }
+    return R;
+}
+
+cudaError_t launch_trace_fp64(const GridDev &g, const FanDev &f, int rays_per_warp, rt_ray_result *out,
+                              cudaStream_t st) {
+    const int R = rays_per_warp;
+    const long long blocks = (f.n_rays + R - 1) / R;
+    trace_fp64_kernel<<<(unsigned)blocks, 32, fp64_smem_bytes(R), st>>>(g, f, R, out);
+    return cudaGetLastError();
+}
+
+}  // namespace rtgd

@@ -63,6 +63,7 @@ struct LaunchPlan {
     int threads;
     int blocks;   // persistent grid size
     int lanes;    // lanes per ray (1, 2, 4)
+    int fp64_rays = 1;   // FP64 path: rays a warp starts with (fp64_rays_per_warp)
     int smem = 0; // plain kernel: dynamic shared memory per block (bytes); see plain_exclusive_smem
     // plain kernel: an event (timing disabled) that the launch records once
     // all of its blocks have begun (a launch-completion event), or null
@@ -72,10 +73,15 @@ struct LaunchPlan {
 cudaError_t launch_grid_prep(const void *raw, int dtype, const GridSizes &sz, double *pad64, float *pad32,
                              float4 *quad, float4 *table, cudaStream_t st);
 cudaError_t upload_tableaus();
-// Trace launch then (mixed path) the pass that turns the raw final states
+// Trace launch then the pass that turns the raw final states
 // into the records' outputs.
 cudaError_t launch_trace(const GridDev &g, const FanDev &f, rt_ray_result *out, unsigned long long *counter,
                          const LaunchPlan &lp, cudaStream_t st);
+// FP64 path: rays per warp at the start for a fan of n_rays on a device with
+// sms SMs, and the launch (raw final states, as the mixed path's).
+int fp64_rays_per_warp(long long n_rays, int sms);
+cudaError_t launch_trace_fp64(const GridDev &g, const FanDev &f, int rays_per_warp, rt_ray_result *out,
+                              cudaStream_t st);
 // The two steps separately (an ordered plan finishes once after its two launches).
 cudaError_t launch_trace_only(const GridDev &g, const FanDev &f, rt_ray_result *out, unsigned long long *counter,
                               const LaunchPlan &lp, cudaStream_t st);

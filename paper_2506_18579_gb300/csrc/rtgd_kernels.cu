@@ -23,6 +23,8 @@
 
 #include "rtgd.h"
 #include "rtgd_device.cuh"
+#include "rtgd_fan.cuh"
+#include "rtgd_fp64.cuh"
 #include "rtgd_internal.h"
 
 namespace rtgd {
@@ -136,73 +138,8 @@ cudaError_t launch_grid_prep(const void *raw, int dtype, const GridSizes &sz, do
     return cudaGetLastError();
 }
 
-// ====================================================================== fan
-// Canonical ray index -> (frequency, mode, elevation, azimuth) of the fan,
-// order [freq][mode][el][az], with the per-fan table entries of each.
-struct RayParams {
-    double f_hz;
-    float xfac, ab0;        // the mixed path's per-frequency factors
-    double se, ce, sa, ca;  // sin, cos of elevation and azimuth
-    double az;              // azimuth (rad)
-    int mode;
-};
-
-// Fans hold fewer than 2^31 rays (checked on the host), so 32-bit index
-// arithmetic suffices (64-bit divisions are long instruction sequences).
-__device__ __forceinline__ RayParams ray_params(const FanDev &f, long long id64) {
-    const unsigned id = (unsigned)id64;
-    const unsigned a = id % (unsigned)f.n_az;
-    const unsigned rest = id / (unsigned)f.n_az;
-    const unsigned e = rest % (unsigned)f.n_el;
-    const unsigned rest2 = rest / (unsigned)f.n_el;
-    const unsigned m = rest2 % (unsigned)f.n_modes;
-    const unsigned q = rest2 / (unsigned)f.n_modes;
-    RayParams p;
-    p.f_hz = f.freq[q].f_hz;
-    p.xfac = f.freq[q].xfac;
-    p.ab0 = f.freq[q].ab0;
-    p.se = f.el[e].s;
-    p.ce = f.el[e].c;
-    p.sa = f.az[a].s;
-    p.ca = f.az[a].c;
-    p.az = f.az[a].rad;
-    p.mode = (m == 0) ? f.mode0 : f.mode1;
-    return p;
-}
-
-// Claim index -> canonical index.  ORDER_ELEVATION_FASTEST hands out
-// neighbouring elevations of one azimuth together (similar paths, so the
-// lanes of a warp gather from nearby cells).
-__device__ __forceinline__ long long claim_to_ray(const FanDev &f, long long c64) {
-    if (f.perm) return f.perm[f.perm_off + c64];
-    if (f.order != RT_ORDER_ELEVATION_FASTEST) return c64;
-    const unsigned c = (unsigned)c64;
-    const unsigned e = c % (unsigned)f.n_el;
-    const unsigned rest = c / (unsigned)f.n_el;
-    const unsigned a = rest % (unsigned)f.n_az;
-    const unsigned fm = rest / (unsigned)f.n_az;  // freq * n_modes + mode
-    return ((long long)fm * f.n_el + e) * f.n_az + a;
-}
-
 // ================================================================ utilities
 __device__ __forceinline__ double wrap180(double x) { return x - 360.0 * floor((x + 180.0) / 360.0); }
-
-// Peak of the cubic Hermite fit of r(s), s in [0,1], through (r0, h d0) and
-// (r1, h d1) with d0 > 0 >= d1 (zero of p'(s) by bisection).
-__device__ double hermite_peak(double r0, double r1, double d0, double d1, double h) {
-    const double m0 = h * d0, m1 = h * d1;
-    const double A = 2.0 * (r0 - r1) + m0 + m1;
-    const double B = 3.0 * (r1 - r0) - 2.0 * m0 - m1;
-    double lo = 0.0, hi = 1.0;
-    for (int it = 0; it < 60; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        const double dp = m0 + 2.0 * B * mid + 3.0 * A * mid * mid;
-        if (dp > 0.0) lo = mid;
-        else hi = mid;
-    }
-    const double s = 0.5 * (lo + hi);
-    return r0 + m0 * s + B * s * s + A * s * s * s;
-}
 
 // Output quantities of a final state (Sec. II-C: group path, ground distance,
 // azimuth deviation, reflection height): central angle and initial bearing
@@ -234,321 +171,12 @@ __device__ __noinline__ void finish_result(double tx_th, double tx_ph, double az
     *out = r;
 }
 
-__device__ __forceinline__ bool finite6(const double y[6]) {
-    bool ok = true;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) ok = ok && isfinite(y[i]);
-    return ok;
-}
-
-// Lateral position inside the grid's lat/lon span?
-__device__ __forceinline__ bool inside_latlon(const GridDev &g, double th, double ph) {
-    const double lat = 90.0 - th * kRad2Deg;
-    double lonrel = ph * kRad2Deg - g.lon0;
-    lonrel -= 360.0 * floor(lonrel / 360.0);
-    const double xa = (lat - g.lat0) * g.inv_dlat;
-    const double xb = lonrel * g.inv_dlon;
-    return xa >= 0.0 && xa <= (double)(g.n_lat - 1) && xb >= 0.0 && xb <= (double)(g.n_lon - 1);
-}
-
-// ================================================================ FP64 path
-// dy/dP' at state y, all in double: Ne and its gradient from the FP64 padded
-// grid (Eq. 13), then the dipole, Appleton-Hartree and Eq. 1.
-__device__ void rhs64(const GridDev &g, const RayPhys<double> &rp, const double y[6], double dy[6],
-                      double *mu2) {
-    StageIn<double> s;
-    s.r = y[0];
-    sincos(y[1], &s.sth, &s.cth);
-    sincos(y[2], &s.sph, &s.cph);
-    s.k[0] = y[3];
-    s.k[1] = y[4];
-    s.k[2] = y[5];
-    const double alt = y[0] - g.R_E;
-    const double lat = 90.0 - y[1] * kRad2Deg;
-    double lonrel = y[2] * kRad2Deg - g.lon0;
-    lonrel -= 360.0 * floor(lonrel / 360.0);
-    const double xa = (lat - g.lat0) * g.inv_dlat;
-    const double xb = lonrel * g.inv_dlon;
-    const double xc = (alt - g.alt0) * g.inv_dalt;
-    int ia, ib, ic;
-    double ta, tb, tc;
-    s.X = 0.0;
-    s.dX[0] = s.dX[1] = s.dX[2] = 0.0;
-    if (cell_coord<double>(xa, g.n_lat, ia, ta) && cell_coord<double>(xb, g.n_lon, ib, tb) &&
-        cell_coord<double>(xc, g.n_alt, ic, tc)) {
-        double wa[4], da[4], wb[4], db[4], wc[4], dc[4], out[4];
-        interp_weights<double>(ta, wa, da, g.interp);
-        interp_weights<double>(tb, wb, db, g.interp);
-        interp_weights<double>(tc, wc, dc, g.interp);
-        const long long sj = g.p_alt, si = (long long)g.p_lon * g.p_alt;
-        // padded index of node (ia-1, ib-1, ic-1) is (ia, ib, ic)
-        const double *base = g.pad64 + (long long)ia * si + (long long)ib * sj + ic;
-#define RTGD_ROW64(a, b, u0, u1, u2, u3)              \
-    {                                                 \
-        const double *p_ = base + (a) * si + (b) * sj; \
-        u0 = __ldg(p_);                               \
-        u1 = __ldg(p_ + 1);                           \
-        u2 = __ldg(p_ + 2);                           \
-        u3 = __ldg(p_ + 3);                           \
-    }
-        RTGD_CONTRACT(double, false, RTGD_ROW64, 0.0, 0, 4, wa, da, wb, db, wc, dc, out);
-#undef RTGD_ROW64
-        s.X = rp.xfac * out[0];
-        s.dX[0] = rp.xfac * out[3] * g.inv_dalt;
-        s.dX[1] = -rp.xfac * out[1] * g.inv_dlat * kRad2Deg;
-        s.dX[2] = rp.xfac * out[2] * g.inv_dlon * kRad2Deg;
-    }
-    const FieldTerms<double> F = field_terms<double>(rp, s);
-    ray_rhs<double>(rp, s, F, dy, mu2);
-}
-
-__device__ void rk4_step64(const GridDev &g, const RayPhys<double> &rp, const double y[6], const double k1[6],
-                           double h, double yn[6]) {
-    double k2[6], k3[6], k4[6], t[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) t[i] = y[i] + 0.5 * h * k1[i];
-    rhs64(g, rp, t, k2, nullptr);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) t[i] = y[i] + 0.5 * h * k2[i];
-    rhs64(g, rp, t, k3, nullptr);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) t[i] = y[i] + h * k3[i];
-    rhs64(g, rp, t, k4, nullptr);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) yn[i] = y[i] + h / 6.0 * (k1[i] + 2.0 * k2[i] + 2.0 * k3[i] + k4[i]);
-}
-
-// Runge-Kutta-Fehlberg 4(5): fourth-order solution in yn, local error
-// estimate (5th - 4th order) in e, formed as h sum((b5_i - b4_i) k_i) so it
-// keeps full relative precision (y5 - y4 would cancel against r ~ 6371 km).
-__device__ void rkf45_step64(const GridDev &g, const RayPhys<double> &rp, const double y[6], const double k1[6],
-                             double h, double yn[6], double e[6]) {
-    double k2[6], k3[6], k4[6], k5[6], k6[6], t[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) t[i] = y[i] + h * (k1[i] / 4.0);
-    rhs64(g, rp, t, k2, nullptr);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) t[i] = y[i] + h * (3.0 / 32.0 * k1[i] + 9.0 / 32.0 * k2[i]);
-    rhs64(g, rp, t, k3, nullptr);
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-        t[i] = y[i] + h * (1932.0 / 2197.0 * k1[i] - 7200.0 / 2197.0 * k2[i] + 7296.0 / 2197.0 * k3[i]);
-    rhs64(g, rp, t, k4, nullptr);
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-        t[i] = y[i] + h * (439.0 / 216.0 * k1[i] - 8.0 * k2[i] + 3680.0 / 513.0 * k3[i] - 845.0 / 4104.0 * k4[i]);
-    rhs64(g, rp, t, k5, nullptr);
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-        t[i] = y[i] + h * (-8.0 / 27.0 * k1[i] + 2.0 * k2[i] - 3544.0 / 2565.0 * k3[i] + 1859.0 / 4104.0 * k4[i] -
-                           11.0 / 40.0 * k5[i]);
-    rhs64(g, rp, t, k6, nullptr);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        yn[i] = y[i] + h * (25.0 / 216.0 * k1[i] + 1408.0 / 2565.0 * k3[i] + 2197.0 / 4104.0 * k4[i] - k5[i] / 5.0);
-        e[i] = h * ((16.0 / 135.0 - 25.0 / 216.0) * k1[i] + (6656.0 / 12825.0 - 1408.0 / 2565.0) * k3[i] +
-                    (28561.0 / 56430.0 - 2197.0 / 4104.0) * k4[i] + (1.0 / 5.0 - 9.0 / 50.0) * k5[i] +
-                    2.0 / 55.0 * k6[i]);
-    }
-}
-
 // RKF45 error norm (<= 1 accepts) and step factor, as documented in rtgd.h.
 template <typename R>
 __device__ __forceinline__ R rkf45_err(R r, R sth, R kmag, const R e[6], R rtol, R atol) {
     const R pos = fmax(fabs(e[0]), fmax(r * fabs(e[1]), r * sth * fabs(e[2])));
     const R kerr = fmax(fabs(e[3]), fmax(fabs(e[4]), fabs(e[5])));
     return fmax(fdiv(pos, atol + rtol * r), fdiv(kerr, rtol * fmax(kmag, R(1e-3))));
-}
-
-// Step-size factor: 0.9 err^(-1/5) limited to [0.2, 5], rounded down to a
-// power of 2^(1/4), so step sizes change through discrete decisions only and
-// round-off in err cannot feed back into the step sequence.
-template <typename R>
-__device__ __forceinline__ double step_factor(R err) {
-    const R fac = (err == R(0)) ? R(5) : fmin(R(5), fmax(R(0.2), R(0.9) * pow(err, R(-0.2))));
-    return exp2(floor(4.0 * log2((double)fac)) * 0.25);
-}
-
-// Launch direction (elevation above the horizontal, azimuth clockwise from
-// north; the theta unit vector points south) and position of a ray, from the
-// fan's sine and cosine tables.
-__device__ __forceinline__ void launch_dir(const FanDev &f, const RayParams &p, double y[6]) {
-    y[0] = f.tx_r;
-    y[1] = f.tx_th;
-    y[2] = f.tx_ph;
-    y[3] = p.se;
-    y[4] = -p.ce * p.ca;
-    y[5] = p.ce * p.sa;
-}
-
-// Group path to the next cell face the ray reaches, predicted linearly from
-// dy/dP' = k1.  Faces are where the C1 interpolant's second derivatives jump
-// (the right-hand side is only C0 there), the grid's outer faces included;
-// lateral faces count only inside the altitude span.  Adaptive steps end just
-// past such a face instead of straddling it.
-__device__ double face_distance64(const GridDev &g, const double y[6], const double k1[6]) {
-    const double lat = 90.0 - y[1] * kRad2Deg;
-    double lonrel = y[2] * kRad2Deg - g.lon0;
-    lonrel -= 360.0 * floor(lonrel * (1.0 / 360.0));
-    const double x[3] = {(lat - g.lat0) * g.inv_dlat, lonrel * g.inv_dlon, (y[0] - g.R_E - g.alt0) * g.inv_dalt};
-    const double v[3] = {-k1[1] * kRad2Deg * g.inv_dlat, k1[2] * kRad2Deg * g.inv_dlon, k1[0] * g.inv_dalt};
-    const int n[3] = {g.n_lat, g.n_lon, g.n_alt};
-    const bool in_alt = x[2] >= 0.0 && x[2] <= (double)(g.n_alt - 1);
-    double best = HUGE_VAL;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        if (a < 2 && !in_alt) continue;
-        if (v[a] > 0.0) {
-            double F = floor(x[a]) + 1.0;
-            if (F < 0.0) F = 0.0;
-            if (F <= (double)(n[a] - 1)) best = fmin(best, (F - x[a]) / v[a]);
-        } else if (v[a] < 0.0) {
-            double F = ceil(x[a]) - 1.0;
-            if (F > (double)(n[a] - 1)) F = (double)(n[a] - 1);
-            if (F >= 0.0) best = fmin(best, (F - x[a]) / v[a]);
-        }
-    }
-    return best;
-}
-
-__device__ void trace_ray_fp64(const GridDev &g, const FanDev &f, long long id, rt_ray_result *out) {
-    const RayParams p = ray_params(f, id);
-    const RayPhys<double> rp = make_phys<double>(g, p.f_hz, p.mode);
-    const double RE = g.R_E;
-    double y[6], dummy[6], mu2 = 0.0;
-    launch_dir(f, p, y);
-    rhs64(g, rp, y, dummy, &mu2);  // mu^2 at the transmitter for this direction
-    if (!(mu2 > 0.0)) {
-        finish_result(f.tx_th, f.tx_ph, p.az, y[1], y[2], 0.0, f.tx_r - RE, RT_RAY_NONFINITE, 0, 0, 1, RE, out);
-        return;
-    }
-    const double mu = sqrt(mu2);
-    y[3] *= mu;
-    y[4] *= mu;
-    y[5] *= mu;
-    const bool adaptive = f.integrator == RT_RKF45;
-    double P = 0.0, h = f.h0, apo = y[0] - RE;
-    int n_steps = 0, n_att = 0, n_ev = 1, status = RT_RAY_NOT_RUN;
-    const int ev_per_step = adaptive ? 5 : 3;  // stage evaluations besides k1
-    bool have_prev = false, k1_valid = false;
-    double r_prev = 0.0, dr_prev = 0.0, h_prev = 0.0;
-    double k1[6];
-    while (status == RT_RAY_NOT_RUN) {
-        if (n_att >= f.max_steps) {
-            status = RT_RAY_MAX_STEPS;
-            break;
-        }
-        double hs = h;
-        if (!k1_valid) {
-            rhs64(g, rp, y, k1, nullptr);
-            k1_valid = true;
-            ++n_ev;
-        }
-        bool at_face = false;
-        if (adaptive) {
-            const double hf = face_distance64(g, y, k1);
-            if (hf > 1e-3 * hs && hf < hs) {
-                hs = hf * (1.0 + 1e-4);
-                at_face = true;
-            }
-        }
-        if (f.max_path > 0.0 && P + hs > f.max_path) hs = f.max_path - P;
-        if (have_prev && dr_prev > 0.0 && k1[0] <= 0.0)
-            apo = fmax(apo, hermite_peak(r_prev, y[0], dr_prev, k1[0], h_prev) - RE);
-        have_prev = false;
-        double yn[6], e[6];
-        if (adaptive) rkf45_step64(g, rp, y, k1, hs, yn, e);
-        else rk4_step64(g, rp, y, k1, hs, yn);
-        ++n_att;
-        n_ev += ev_per_step;
-        double h_next = h;
-        if (adaptive) {
-            const double err = rkf45_err<double>(y[0], sin(y[1]), sqrt(y[3] * y[3] + y[4] * y[4] + y[5] * y[5]), e,
-                                                 f.rtol, f.atol);
-            const double fac = step_factor<double>(err);
-            // the nominal step changes only by quantised factors of itself
-            if (!(err <= 1.0)) {
-                h = h * fac;
-                if (h < f.hmin) status = RT_RAY_STEP_UNDERFLOW;
-                continue;
-            }
-            h_next = fmin(fmax(h * (at_face ? fmin(1.0, fac) : fac), f.hmin), f.hmax);
-        }
-        if (!finite6(yn)) {
-            status = RT_RAY_NONFINITE;
-            break;
-        }
-        const bool lands = yn[0] < RE;
-        const bool exits = !lands && yn[0] - RE > g.top;
-        if (lands || exits) {
-            // ground return or exit through the grid top inside this step:
-            // r(step(h*)) = R_E (or R_E + top) for h* in (0, hs], Illinois regula
-            // falsi; sg makes the bracket function positive at the step start
-            const double rt = lands ? RE : RE + g.top, sg = lands ? 1.0 : -1.0;
-            double a = 0.0, fa = sg * (y[0] - rt), b = hs, fb = sg * (yn[0] - rt), c = b;
-            double yc[6], ec[6];
-#pragma unroll
-            for (int i = 0; i < 6; ++i) yc[i] = yn[i];
-            int side = 0;
-            for (int it = 0; it < 60; ++it) {
-                c = b - fb * (b - a) / (fb - fa);
-                if (adaptive) rkf45_step64(g, rp, y, k1, c, yc, ec);
-                else rk4_step64(g, rp, y, k1, c, yc);
-                ++n_att;
-                n_ev += ev_per_step;
-                const double fc = sg * (yc[0] - rt);
-                if (fabs(fc) < 1e-9) break;
-                if (fc < 0.0) {
-                    b = c;
-                    fb = fc;
-                    if (side == -1) fa *= 0.5;
-                    side = -1;
-                } else {
-                    a = c;
-                    fa = fc;
-                    if (side == 1) fb *= 0.5;
-                    side = 1;
-                }
-            }
-            P += c;
-            ++n_steps;
-#pragma unroll
-            for (int i = 0; i < 6; ++i) y[i] = yc[i];
-            if (exits) apo = fmax(apo, y[0] - RE);
-            status = lands ? RT_RAY_LANDED : RT_RAY_ESCAPED;
-            break;
-        }
-        P += hs;
-        ++n_steps;
-        apo = fmax(apo, yn[0] - RE);
-        have_prev = true;
-        r_prev = y[0];
-        dr_prev = k1[0];
-        h_prev = hs;
-#pragma unroll
-        for (int i = 0; i < 6; ++i) y[i] = yn[i];
-        k1_valid = false;
-        const double alt = y[0] - RE;
-        if (alt >= g.alt0 && !inside_latlon(g, y[1], y[2])) {
-            status = RT_RAY_LEFT_GRID;
-            break;
-        }
-        if (f.max_path > 0.0 && P >= f.max_path - 1e-12) {
-            status = RT_RAY_MAX_PATH;
-            break;
-        }
-        h = h_next;
-    }
-    finish_result(f.tx_th, f.tx_ph, p.az, y[1], y[2], P, apo, status, n_steps, n_att, n_ev, RE, out);
-}
-
-__global__ void __launch_bounds__(128) trace_fp64_kernel(GridDev g, FanDev f, rt_ray_result *__restrict__ out) {
-    const long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (id >= f.n_rays) return;
-    const long long ray = claim_to_ray(f, id);
-    rt_ray_result r;
-    trace_ray_fp64(g, f, ray, &r);
-    out[ray] = r;
 }
 
 // =============================================================== mixed path
@@ -1769,12 +1397,7 @@ static cudaError_t launch_mixed(const GridDev &g, const FanDev &f, rt_ray_result
 cudaError_t launch_trace_only(const GridDev &g, const FanDev &f, rt_ray_result *out, unsigned long long *counter,
                               const LaunchPlan &lp, cudaStream_t st) {
     if (f.n_rays == 0) return cudaSuccess;
-    if (f.precision == RT_FP64) {
-        const int threads = 128;
-        const long long blocks = (f.n_rays + threads - 1) / threads;
-        trace_fp64_kernel<<<(unsigned)blocks, threads, 0, st>>>(g, f, out);
-        return cudaGetLastError();
-    }
+    if (f.precision == RT_FP64) return launch_trace_fp64(g, f, lp.fp64_rays, out, st);
     switch (lp.stencil) {
         case RT_STENCIL_GATHER: return launch_mixed<RT_STENCIL_GATHER>(g, f, out, counter, lp, st);
         case RT_STENCIL_TABLE: return launch_mixed<RT_STENCIL_TABLE>(g, f, out, counter, lp, st);
@@ -1783,7 +1406,7 @@ cudaError_t launch_trace_only(const GridDev &g, const FanDev &f, rt_ray_result *
 }
 
 cudaError_t launch_finish(const GridDev &g, const FanDev &f, rt_ray_result *out, long long n, cudaStream_t st) {
-    if (f.precision == RT_FP64 || n == 0) return cudaSuccess;  // the FP64 kernel writes final records itself
+    if (n == 0) return cudaSuccess;
     const int threads = 128;
     finish_records_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0, st>>>(g.R_E, f, out, n);
     return cudaGetLastError();
