@@ -294,29 +294,24 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float d) {
 
 // Stage cell along one axis from base cell i0 and offset coordinate t = t0 +
 // delta * scale; false outside [0, n-1], and then cell 0 at t = 0, so that the
-// caller can gather from an in-bounds cell without branching.
+// caller can gather from an in-bounds cell without branching.  On the critical
+// path of every stage, so floor(t) costs one addition: t + 1.5 * 2^23 rounded
+// down holds it in the low mantissa bits.  That is exact for |t| < 2^22; beyond
+// that, and for NaN, the integer lands at least 2^22 cells out, which the index
+// test refuses (base cells lie within +-10^6 of the grid, grids have fewer
+// nodes per axis than that).  Nine instructions; with a clamp and a
+// round-to-nearest that was corrected afterwards it took sixteen.
 __device__ __forceinline__ bool stage_cell(int i0, float t, int n, int &i, float &tt) {
-    // floor of t clamped to +-1e6 (keeps the int sum far from overflow) without
-    // conversion instructions: adding 1.5 * 2^23 rounds to the nearest integer,
-    // which sits in the low mantissa bits; one less if that rounded up.  A NaN
-    // t clamps to -1e6 and then fails the cell index test below.
     const float magic = 12582912.0f;
-    const float tc = fminf(fmaxf(t, -1e6f), 1e6f);
-    const float big = tc + magic;
-    const float near = big - magic;
-    const bool up = near > tc;
-    const float fl = up ? near - 1.0f : near;
-    int ii = i0 + (__float_as_int(big) - __float_as_int(magic)) - (up ? 1 : 0);
-    float tr = t - fl;
+    const float big = __fadd_rd(t, magic);
+    const int ii = (int)((unsigned)i0 + (unsigned)__float_as_int(big) - (unsigned)__float_as_int(magic));
+    const float tr = t - (big - magic);
     const bool last = (ii == n - 1) & (tr == 0.0f);  // the last node: cell n-2 at t = 1
-    ii = last ? n - 2 : ii;
-    tr = last ? 1.0f : tr;
-    // tr = t - floor(t) lies in [0, 1] by construction, so the cell index alone
-    // decides; a NaN or an offset beyond the clamp puts it ~1e6 cells out
+    // tr = t - floor(t) lies in [0, 1] by construction, so the cell index alone decides
     const bool ok = (unsigned)ii < (unsigned)(n - 1);
-    i = ok ? ii : 0;
-    tt = ok ? tr : 0.0f;
-    return ok;
+    i = last ? n - 2 : (ok ? ii : 0);
+    tt = last ? 1.0f : (ok ? tr : 0.0f);
+    return ok | last;
 }
 
 // Lat-weights of the rows a = q*4/G .. (q+1)*4/G - 1 handled by lane q of a
@@ -343,6 +338,14 @@ __device__ __forceinline__ void own_lat_weights(float ta, int q, float wa[4], fl
     }
 }
 
+// Index of (i, j, k) in an array of rows of n_k entries, n_j rows per i: the
+// row number in 32 bits (a grid with 2^32 (lat, lon) rows of four samples
+// would not fit the device), then one wide multiply-add.
+__device__ __forceinline__ unsigned long long row_index(int i, int n_j, int j, int n_k, int k) {
+    const unsigned row = (unsigned)i * (unsigned)n_j + (unsigned)j;
+    return (unsigned long long)row * (unsigned)n_k + (unsigned)k;
+}
+
 // dy/dP' (float) at base + delta.  STENCIL selects where the 64 samples come
 // from and IP the interpolant (0 GD, 1 Catmull-Rom); with G > 1 the G lanes
 // of a group (lane q, shuffle mask gmask) split the 16 sample rows and combine
@@ -366,10 +369,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
     const bool in_a = stage_cell(b.ia, b.ta + g.sa * d[1], g.n_lat, ia, ta);
     const bool in_b = stage_cell(b.ib, b.tb + g.sb * d[2], g.n_lon, ib, tb);
     const bool in_c = stage_cell(b.ic, b.tc + g.sc * d[0], g.n_alt, ic, tc);
-    const bool inside = in_a & in_b & in_c;
-    ia = inside ? ia : 0;
-    ib = inside ? ib : 0;
-    ic = inside ? ic : 0;
+    const bool inside = in_a & in_b & in_c;  // each axis is in bounds by itself
     float wa[4], da[4], wb[4], db[4], wc[4], dc[4], out[4], ref;
     constexpr int NA = 4 / G;
     const int a0 = q * NA;
@@ -379,7 +379,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
     if (STENCIL == RT_STENCIL_QUAD) {
         // quad (pi, pj, k): 4 samples of cell k in padded row (pi, pj); node i-1 -> padded i
         const long long sj = g.q_alt, si = (long long)(g.n_lon + 2) * g.q_alt;
-        const float4 *qp = g.quad + (long long)ia * si + (long long)ib * sj + ic;
+        const float4 *qp = g.quad + row_index(ia, g.n_lon + 2, ib, g.q_alt, ic);
         ref = __ldg(qp + si + sj).y;  // node (ia, ib, ic)
 #define RTGD_ROWQ(a, b, u0, u1, u2, u3)                    \
     {                                                      \
@@ -392,9 +392,15 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
         RTGD_CONTRACT(float, (G > 1), RTGD_ROWQ, ref, a0, NA, wa, da, wb, db, wc, dc, out);
 #undef RTGD_ROWQ
     } else if (STENCIL == RT_STENCIL_TABLE) {
-        const long long cell = ((long long)ia * (g.n_lon - 1) + ib) * (g.n_alt - 1) + ic;
+        // one lane per ray: products in 64 bits.  Fewer instructions through
+        // row_index, but the one-lane loop then schedules its 17 loads worse
+        // (495,122 rays 71.6 against 65.6 ms); several lanes gain (C2 fan at four
+        // lanes 11.75 against 11.9 ms)
+        const long long cell = G == 1 ? ((long long)ia * (g.n_lon - 1) + ib) * (g.n_alt - 1) + ic
+                                      : (long long)row_index(ia, g.n_lon - 1, ib, g.q_alt, ic);
         const float4 *qp = g.table + cell * 16;  // samples minus the node (ia, ib, ic)
-        ref = __ldg(g.pad32 + (long long)(ia + 1) * g.p_lon * g.p_alt + (long long)(ib + 1) * g.p_alt + ic + 1);
+        ref = __ldg(g.pad32 + (G == 1 ? (long long)(ia + 1) * g.p_lon * g.p_alt + (long long)(ib + 1) * g.p_alt + ic + 1
+                                      : (long long)row_index(ia + 1, g.p_lon, ib + 1, g.p_alt, ic + 1)));
 #define RTGD_ROWT(a, b, u0, u1, u2, u3)              \
     {                                                \
         const float4 v_ = __ldg(qp + (a) * 4 + (b)); \
@@ -407,7 +413,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
 #undef RTGD_ROWT
     } else {
         const long long sj = g.p_alt, si = (long long)g.p_lon * g.p_alt;
-        const float *p = g.pad32 + (long long)ia * si + (long long)ib * sj + ic;
+        const float *p = g.pad32 + row_index(ia, g.p_lon, ib, g.p_alt, ic);
         ref = __ldg(p + si + sj + 1);  // node (ia, ib, ic)
 #define RTGD_ROWG(a, b, u0, u1, u2, u3)            \
     {                                              \
