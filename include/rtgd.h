@@ -194,7 +194,8 @@ typedef struct rt_launch_config {
                               groups (the default); PERSISTENT = one resident grid whose lane
                               groups claim rays from an atomic counter (mixed only) */
     int32_t stencil;       /* RT_STENCIL_*: where the mixed path reads the 4x4x4 samples:
-                              GATHER = padded FP32 grid, QUAD = 4 consecutive altitude samples
+                              GATHER = padded FP32 grid (persistent kernel; the plain kernels read
+                              the same samples from the QUAD layout), QUAD = 4 consecutive altitude samples
                               per float4, TABLE = per-cell table (needs RT_GRID_TABLE) */
     int32_t block_threads; /* 0 = default (128); a multiple of 32 in [32, 128] */
     int32_t order;         /* RT_ORDER_*: order in which rays are handed to lane groups (both

@@ -37,7 +37,7 @@ struct GridDev {
     double m[3];                     // unit vector to the geomagnetic north pole
     float sa, sb, sc;                // d(grid coord)/d(theta, phi, r): -rad2deg/dlat, rad2deg/dlon, 1/dalt
     float R_Ef, mf[3];               // float copies of R_E and m
-    float top_f;                     // top as float
+    float top_f, alt0_f;             // top and alt0 as floats
     int iso;                         // no field (b0 == 0)
     int interp;                      // 0: Galerkin-Difference p=3, 1: Catmull-Rom (comparison)
     const double *pad64;             // (n_lat+2)(n_lon+2)(n_alt+2) doubles

@@ -205,45 +205,65 @@ struct Base32 {
     float k[3];
 };
 
-// 2^(k/4) for k = -10..9: the quantised step factors (see step_factor).
-__constant__ float c_pow2q[20];
+// (double)x and (float)x by integer operations: a conversion is an FP64-rate
+// instruction (64 cycles of a warp on GB300), these are ~8 integer ones.
+// Zeros, subnormals, infinities, NaN and doubles outside the normal float
+// range take the conversion.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u) return (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ float narrow(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffull;
+    const unsigned e = (unsigned)(m >> 52);
+    if (e - 897u >= 253u) return (float)x;  // exponents 897..1149: normal floats, rounding cannot overflow
+    const unsigned long long r = m - (896ull << 52) + 0x0fffffffull + ((m >> 29) & 1ull);  // to nearest, ties to even
+    return __uint_as_float((unsigned)(r >> 29) | ((unsigned)(b >> 32) & 0x80000000u));
+}
 
-__device__ __forceinline__ int clamp_cell(double f) { return (int)fmin(fmax(f, -1e6), 1e6); }
+// floor(x) as an integer and the fraction x - floor(x): one addition rounded
+// down, exact for |x| < 2^31.  Beyond +-10^6 (and for NaN) the cell is clamped
+// to that (negative side for NaN), which stays outside of the grid.
+__device__ __forceinline__ int floor_cell(double x, float &t) {
+    const double magic = 6755399441055744.0;  // 1.5 * 2^52
+    const double big = __dadd_rd(x, magic);
+    const double fl = big - magic;
+    const int hi = __double2hiint(x) & 0x7fffffff;
+    t = narrow(x - fl);
+    if (hi < 0x412e8480) return __double2loint(big);  // |x| < 10^6
+    const double f = floor(x);
+    t = (float)(x - f);
+    return (int)fmin(fmax(f, -1e6), 1e6);
+}
 
 // Base of a double state (double arithmetic; used at launch and to resync).
 // Out of line with scalar arguments (it runs at launch and every kResyncSteps
-// accepted steps), returning the base by value.
+// accepted steps), returning the base by value; the caller sets the wave
+// vector.  The rays of a warp resync at different steps, so almost every
+// attempt of a full warp waits for this once: 17 FP64 instructions (a further
+// 8 in lane_fold), where floors, clamps, conversions and a division-free wrap
+// in FP64 made it ~65.
 __device__ __noinline__ Base32 base_of(double lat0, double lon0, double inv_dlat, double inv_dlon, double R_E,
-                                       double alt0, double inv_dalt, double r, double th, double ph, double k0,
-                                       double k1, double k2) {
+                                       double alt0, double inv_dalt, double r, double th, double ph) {
     Base32 b;
     const double lat = 90.0 - th * kRad2Deg;
-    double lonrel = ph * kRad2Deg - lon0;
-    lonrel -= 360.0 * floor(lonrel * (1.0 / 360.0));
-    const double xa = (lat - lat0) * inv_dlat;
-    const double xb = lonrel * inv_dlon;
-    const double xc = (r - R_E - alt0) * inv_dalt;
-    const double fa = floor(xa), fb = floor(xb), fc = floor(xc);
-    // positions far outside the grid are clamped so the integer stays small; they
-    // remain outside (and non-finite positions give NaN fractions, also outside)
-    b.ia = clamp_cell(fa);
-    b.ib = clamp_cell(fb);
-    b.ic = clamp_cell(fc);
-    b.ta = (float)(xa - fa);
-    b.tb = (float)(xb - fb);
-    b.tc = (float)(xc - fc);
-    b.r = (float)r;
-    b.alt = (float)(r - R_E);
-    sincosf((float)th, &b.sth, &b.cth);
-    sincosf((float)ph, &b.sph, &b.cph);
-    b.k[0] = (float)k0;
-    b.k[1] = (float)k1;
-    b.k[2] = (float)k2;
+    const double lonrel = wrap360(ph * kRad2Deg - lon0);
+    const double alt = r - R_E;
+    b.ia = floor_cell((lat - lat0) * inv_dlat, b.ta);
+    b.ib = floor_cell(lonrel * inv_dlon, b.tb);
+    b.ic = floor_cell((alt - alt0) * inv_dalt, b.tc);
+    b.r = narrow(r);
+    b.alt = narrow(alt);
+    sincosf(narrow(th), &b.sth, &b.cth);
+    sincosf(narrow(ph), &b.sph, &b.cph);
     return b;
 }
 
 __device__ __forceinline__ void base_from_state(const GridDev &g, const double y[6], Base32 &b) {
-    b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, y[0], y[1], y[2], y[3], y[4], y[5]);
+    b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, y[0], y[1], y[2]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) b.k[i] = (float)y[3 + i];
 }
 
 __device__ __forceinline__ void shift_axis(int &i, float &t, float dt) {
@@ -456,12 +476,22 @@ struct Tableau {
 
 __constant__ Tableau c_tab[2];  // [RT_RK4], [RT_RKF45]
 
-// Quantised step factor in float (the mixed path's counterpart of step_factor).
+// Quantised step factor in float (the mixed path's counterpart of
+// step_factor64): 2^(k/4), k = floor(4 log2 of the limited 0.9 err^(-1/5)).
+// One logarithm gives that exponent to ~1e-5; within 1e-3 of an integer (and
+// for err = 0, infinite or NaN) the factor itself decides.
 __device__ __forceinline__ float step_factor_f(float err) {
-    const float fac = (err == 0.0f) ? 5.0f : fminf(5.0f, fmaxf(0.2f, 0.9f * __powf(err, -0.2f)));
-    int k = (int)floorf(4.0f * __log2f(fac));
+    const float l = -0.608012374f - 0.8f * __log2f(err);  // 4 log2(0.9 err^-0.2)
+    const float fl = floorf(l), d = l - fl;
+    int k = (int)fl;
+    if (!(d > 1e-3f && d < 0.999f)) {
+        const float fac = (err == 0.0f) ? 5.0f : fminf(5.0f, fmaxf(0.2f, 0.9f * __powf(err, -0.2f)));
+        k = (int)floorf(4.0f * __log2f(fac));
+    }
     k = k < -10 ? -10 : (k > 9 ? 9 : k);
-    return c_pow2q[k + 10];
+    // 2^(k/4): the mantissa of 2^0, 2^(1/4), 2^(1/2) or 2^(3/4) and the exponent floor(k/4)
+    const int m = (k & 2) ? ((k & 1) ? 0x3fd744fd : 0x3fb504f3) : ((k & 1) ? 0x3f9837f0 : 0x3f800000);
+    return __int_as_float(m + ((k >> 2) << 23));
 }
 
 // Peak rise of the cubic Hermite fit over one step, relative to its start:
@@ -478,30 +508,25 @@ __device__ __noinline__ float hermite_rise_f(float dr, float m0, float m1) {  //
     return s * (m0 + s * (B + s * A));
 }
 
-// Float counterpart of face_distance64 on the base's (cell, fraction) grid
+// Float counterpart of face_axis64 on the base's (cell, fraction) grid
 // coordinates: the distance to the next face is (integer - fraction) / rate.
+// Without branches: the three axes' quotients overlap, and the rays of a warp
+// head in different directions (with branches on the signs it took 670 cycles
+// of a lone warp's 7,600 per attempt).
 __device__ __forceinline__ float face_axis_f(int i, float t, int n, float v) {
-    if (v > 0.0f) {
-        int F = i + 1;
-        if (F < 0) F = 0;
-        return F <= n - 1 ? fdiv((float)(F - i) - t, v) : INFINITY;
-    }
-    if (v < 0.0f) {
-        int F = t > 0.0f ? i : i - 1;
-        if (F > n - 1) F = n - 1;
-        return F >= 0 ? fdiv((float)(F - i) - t, v) : INFINITY;
-    }
-    return INFINITY;
+    const bool up = v > 0.0f;
+    const int F = up ? max(i + 1, 0) : min(t > 0.0f ? i : i - 1, n - 1);
+    const bool ok = up ? F <= n - 1 : (v < 0.0f && F >= 0);
+    const float d = fdiv((float)(F - i) - t, v);
+    return ok ? d : INFINITY;
 }
 
 __device__ __forceinline__ float face_distance_f(const GridDev &g, const Base32 &b, const float k1[6]) {
-    float best = face_axis_f(b.ic, b.tc, g.n_alt, g.sc * k1[0]);
-    const bool in_alt = b.ic >= 0 && (b.ic < g.n_alt - 1 || (b.ic == g.n_alt - 1 && b.tc == 0.0f));
-    if (in_alt) {
-        best = fminf(best, face_axis_f(b.ia, b.ta, g.n_lat, g.sa * k1[1]));
-        best = fminf(best, face_axis_f(b.ib, b.tb, g.n_lon, g.sb * k1[2]));
-    }
-    return best;
+    const float c = face_axis_f(b.ic, b.tc, g.n_alt, g.sc * k1[0]);
+    const float l = fminf(face_axis_f(b.ia, b.ta, g.n_lat, g.sa * k1[1]), face_axis_f(b.ib, b.tb, g.n_lon, g.sb * k1[2]));
+    // lateral faces count only inside the altitude span
+    const bool in_alt = (unsigned)b.ic < (unsigned)(g.n_alt - 1) || (b.ic == g.n_alt - 1 && b.tc == 0.0f);
+    return in_alt ? fminf(c, l) : c;
 }
 
 // Per-lane state of the mixed tracer.
@@ -581,8 +606,9 @@ __device__ __forceinline__ void accumulate_next(Lane &L, const Tableau &T, int s
 // Base of the transmitter position (the launch state of every ray of the
 // fan; the wave vector part is set per ray).
 __device__ __forceinline__ Base32 tx_base(const GridDev &g, const FanDev &f) {
-    return base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, f.tx_r, f.tx_th, f.tx_ph, 0.0,
-                   0.0, 0.0);
+    Base32 b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, f.tx_r, f.tx_th, f.tx_ph);
+    b.k[0] = b.k[1] = b.k[2] = 0.0f;
+    return b;
 }
 
 // Starts ray `id`: per-ray constants from the fan's tables, FP64 launch
@@ -629,10 +655,10 @@ __device__ void lane_begin_ray(Lane &L, const GridDev &g, const FanDev &f, long 
 __device__ __forceinline__ void lane_fold(Lane &L) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        L.y[i] += (double)L.inc_hi[i] + (double)L.inc_lo[i];
+        L.y[i] += widen(L.inc_hi[i]) + widen(L.inc_lo[i]);
         L.inc_hi[i] = L.inc_lo[i] = 0.0f;
     }
-    L.P += (double)L.inc_hi[3] + (double)L.inc_lo[3];
+    L.P += widen(L.inc_hi[3]) + widen(L.inc_lo[3]);
     L.inc_hi[3] = L.inc_lo[3] = 0.0f;
 }
 
@@ -908,13 +934,21 @@ __device__ bool lane_end_attempt(Lane &L, const GridDev &g, const FanDev &f, Lan
         L.status = L.exiting ? RT_RAY_ESCAPED : RT_RAY_LANDED;
         return true;
     }
-    float h_next = L.h;
+    float fac = 1.0f;
+    bool accept = true;
     if (f.integrator == RT_RKF45) {
         const float kmag = fsqrt(L.b.k[0] * L.b.k[0] + L.b.k[1] * L.b.k[1] + L.b.k[2] * L.b.k[2]);
         const float err = rkf45_err<float>(L.b.r, L.b.sth, kmag, ef, f.rtol_f, f.atol_f);
-        const float fac = step_factor_f(err);
-        // the nominal step changes only by quantised factors of itself
-        if (!(err <= 1.0f)) {
+        fac = step_factor_f(err);
+        accept = err <= 1.0f;
+    }
+    const float alt_new = L.b.alt + dy4[0];
+    const bool lands = alt_new < 0.0f;
+    // one branch for everything but an accepted step, so that the usual path
+    // below is one block
+    if (!(accept && fin) || lands || alt_new > g.top_f) {
+        if (!accept) {
+            // the nominal step changes only by quantised factors of itself
             L.h = L.h * fac;
             if (L.h < f.hmin_f) {
                 L.status = RT_RAY_STEP_UNDERFLOW;
@@ -922,15 +956,10 @@ __device__ bool lane_end_attempt(Lane &L, const GridDev &g, const FanDev &f, Lan
             }
             return !lane_next_attempt(L, f);
         }
-        h_next = fminf(fmaxf(L.h * (L.at_face ? fminf(1.0f, fac) : fac), f.hmin_f), f.hmax_f);
-    }
-    if (!fin) {
-        L.status = RT_RAY_NONFINITE;
-        return true;
-    }
-    const float alt_new = L.b.alt + dy4[0];
-    const bool lands = alt_new < 0.0f;
-    if (lands || alt_new > g.top_f) {
+        if (!fin) {
+            L.status = RT_RAY_NONFINITE;
+            return true;
+        }
         // ground return or exit through the grid top inside this step
         lane_fold(L);
         const double r_new = L.y[0] + (double)dy4[0];
@@ -947,6 +976,8 @@ __device__ bool lane_end_attempt(Lane &L, const GridDev &g, const FanDev &f, Lan
         L.hs = (float)bracket_first(ls.lb, ls.lfa, ls.lfb);
         return !lane_next_attempt(L, f);
     }
+    if (f.integrator == RT_RKF45)
+        L.h = fminf(fmaxf(L.h * (L.at_face ? fminf(1.0f, fac) : fac), f.hmin_f), f.hmax_f);
     L.r_prev = L.b.r;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -963,19 +994,17 @@ __device__ bool lane_end_attempt(Lane &L, const GridDev &g, const FanDev &f, Lan
     if (++L.since_sync >= kResyncSteps) {
         L.since_sync = 0;
         lane_fold(L);
-        double y[6];
-        lane_state(L, y);
-        base_from_state(g, y, L.b);
+        L.b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, L.y[0], L.y[1], L.y[2]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) L.b.k[i] = L.k_hi[i] + L.k_lo[i];
     } else {
         advance_base(g, L.b, dy4, L.k_hi);
     }
-    if (L.b.alt >= (float)g.alt0) {
-        const bool in_lat = L.b.ia >= 0 && (L.b.ia < g.n_lat - 1 || (L.b.ia == g.n_lat - 1 && L.b.ta == 0.0f));
-        const bool in_lon = L.b.ib >= 0 && (L.b.ib < g.n_lon - 1 || (L.b.ib == g.n_lon - 1 && L.b.tb == 0.0f));
-        if (!(in_lat && in_lon)) {
-            L.status = RT_RAY_LEFT_GRID;
-            return true;
-        }
+    const bool in_lat = (unsigned)L.b.ia < (unsigned)(g.n_lat - 1) || (L.b.ia == g.n_lat - 1 && L.b.ta == 0.0f);
+    const bool in_lon = (unsigned)L.b.ib < (unsigned)(g.n_lon - 1) || (L.b.ib == g.n_lon - 1 && L.b.tb == 0.0f);
+    if (L.b.alt >= g.alt0_f && !(in_lat && in_lon)) {
+        L.status = RT_RAY_LEFT_GRID;
+        return true;
     }
     if (f.has_max_path) {
         lane_fold(L);
@@ -984,7 +1013,6 @@ __device__ bool lane_end_attempt(Lane &L, const GridDev &g, const FanDev &f, Lan
             return true;
         }
     }
-    L.h = h_next;
     return !lane_next_attempt(L, f);
 }
 
@@ -1308,11 +1336,7 @@ static void fill_tableaus(Tableau tab[2]) {
 cudaError_t upload_tableaus() {
     Tableau tab[2];
     fill_tableaus(tab);
-    cudaError_t e = cudaMemcpyToSymbol(c_tab, tab, sizeof(tab));
-    if (e != cudaSuccess) return e;
-    float q[20];
-    for (int k = -10; k <= 9; ++k) q[k + 10] = (float)std::exp2(k * 0.25);
-    return cudaMemcpyToSymbol(c_pow2q, q, sizeof(q));
+    return cudaMemcpyToSymbol(c_tab, tab, sizeof(tab));
 }
 
 template <int STENCIL, int G, int IP>
@@ -1320,6 +1344,8 @@ static cudaError_t launch_mixed_gi(const GridDev &g, const FanDev &f, rt_ray_res
                                    unsigned long long *counter, const LaunchPlan &lp, cudaStream_t st) {
     if (lp.kernel == RT_KERNEL_PERSISTENT) {
         trace_mixed_persistent_kernel<STENCIL, G, IP><<<lp.blocks, lp.threads, 0, st>>>(g, f, out, counter);
+    } else if constexpr (STENCIL == RT_STENCIL_GATHER) {
+        return cudaErrorInvalidValue;  // plain launches read the quad layout instead (make_plan)
     } else {
         const long long blocks = (f.n_rays * G + lp.threads - 1) / lp.threads;
         if (lp.started) {
@@ -1377,7 +1403,6 @@ static cudaError_t exclusive_smem_s(int lanes, int interp, int *bytes) {
 
 cudaError_t plain_exclusive_smem(const LaunchPlan &lp, int interp, int *bytes) {
     switch (lp.stencil) {
-        case RT_STENCIL_GATHER: return exclusive_smem_s<RT_STENCIL_GATHER>(lp.lanes, interp, bytes);
         case RT_STENCIL_TABLE: return exclusive_smem_s<RT_STENCIL_TABLE>(lp.lanes, interp, bytes);
         default: return exclusive_smem_s<RT_STENCIL_QUAD>(lp.lanes, interp, bytes);
     }
@@ -1442,9 +1467,6 @@ cudaError_t launch_trace_fans(const GridDev &g, const FanDev *fans, const long l
     if (n_total == 0) return cudaSuccess;
     cudaError_t e;
     switch (lp.stencil) {
-        case RT_STENCIL_GATHER:
-            e = launch_fans_s<RT_STENCIL_GATHER>(g, fans, first, n_fans, n_total, integrator, out, lp.threads, st);
-            break;
         case RT_STENCIL_TABLE:
             e = launch_fans_s<RT_STENCIL_TABLE>(g, fans, first, n_fans, n_total, integrator, out, lp.threads, st);
             break;
