@@ -65,6 +65,8 @@ static_assert(kSlot % 2 == 1 && cGroup % 2 == 1, "odd strides spread the groups 
 constexpr int kMaxRays = 8;  // rays a warp starts with at most (G = 4)
 constexpr int kPoly = 4 * 5, kPow2 = 20;  // tables at the start of the shared memory
 
+__device__ __noinline__ double div_rare(double x, double c) { return x / c; }
+
 // x / c for a constant c with rc = 1/c correctly rounded: one Newton
 // correction of x rc gives the correctly rounded quotient (Markstein's
 // theorem), 3 FP64 instructions instead of ~10.  Non-finite and tiny x take
@@ -73,13 +75,17 @@ __device__ __forceinline__ double div_const(double x, double c, double rc) {
     const double q = x * rc;
     const double r = fma(-c, q, x);
     const double d = fma(r, rc, q);
-    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
-    return e - 128u < 1800u || (__double2hiint(x) & 0x7fffffff) == 0 ? d : x / c;
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    if ((hi >> 20) - 128u >= 1800u && hi != 0) return div_rare(x, c);
+    return d;
 }
 
 __device__ __forceinline__ bool finite64(double x) {
     return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
 }
+
+// The same with NaN among them: fmax, which ignores a NaN.
+__device__ __noinline__ double max3_rare(double a, double b, double c) { return fmax(fabs(a), fmax(fabs(b), fabs(c))); }
 
 // max of two numbers at least one of which is >= +0 (not NaN): the order of
 // such doubles is the order of their bits as signed integers.
@@ -560,8 +566,8 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
                 pos = max_bits(fabs(e0), max_bits(r * fabs(e1), r * sth * fabs(e2)));
                 kerr = max_bits(fabs(e3), max_bits(fabs(e4), fabs(e5)));
             } else {
-                pos = fmax(fabs(e0), fmax(r * fabs(e1), r * sth * fabs(e2)));
-                kerr = fmax(fabs(e3), fmax(fabs(e4), fabs(e5)));
+                pos = max3_rare(e0, r * e1, r * sth * e2);
+                kerr = max3_rare(e3, e4, e5);
             }
             const double dp = f.atol + f.rtol * r, dk = f.rtol * fmax(kmag, 1e-3);
             const double v = ((q & 1) ? kerr : pos) / ((q & 1) ? dk : dp);

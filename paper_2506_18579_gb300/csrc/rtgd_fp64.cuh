@@ -6,6 +6,11 @@
 
 namespace rtgd {
 
+// Rare cases are out of line here and below: inlined, the compiler predicates
+// them, and a predicated-off FP64 instruction still occupies the warp for its
+// 64 cycles.
+static __device__ __noinline__ double wrap360_rare(double x) { return x - 360.0 * floor(x / 360.0); }
+
 // x - 360 floor(x / 360): the longitude offset wrapped to [0, 360).  The two
 // ranges a ray's longitude lies in are told apart by the high word (a double
 // division costs a warp ~10 FP64 instructions, an integer compare none):
@@ -13,9 +18,9 @@ namespace rtgd {
 // 0; for -360 < x < 0 it is -1.
 __device__ __forceinline__ double wrap360(double x) {
     const unsigned hi = (unsigned)__double2hiint(x);
-    if (hi < 0x40768000u) return x;                                // [0, 360)
-    if (hi >= 0x80100000u && hi < 0xC0768000u) return x + 360.0;   // (-360, 0), normal numbers
-    return x - 360.0 * floor(x / 360.0);
+    if (hi < 0x40768000u) return x;  // [0, 360)
+    if (hi - 0x80100000u < 0xC0768000u - 0x80100000u) return x + 360.0;  // (-360, 0), normal numbers
+    return wrap360_rare(x);
 }
 
 // Grid coordinate of a position along one axis (0 latitude, 1 longitude, 2

@@ -205,36 +205,42 @@ struct Base32 {
     float k[3];
 };
 
+__device__ __noinline__ double widen_rare(float x) { return (double)x; }
+__device__ __noinline__ float narrow_rare(double x) { return (float)x; }
+
 // (double)x and (float)x by integer operations: a conversion is an FP64-rate
 // instruction (64 cycles of a warp on GB300), these are ~8 integer ones.
-// Zeros, subnormals, infinities, NaN and doubles outside the normal float
-// range take the conversion.
+// Subnormals, infinities, NaN and doubles outside the normal float range take
+// the conversion, out of line (see wrap360_rare).
 __device__ __forceinline__ double widen(float x) {
     const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-    if (m - 0x00800000u >= 0x7f000000u) return (double)x;
-    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+    if (m - 0x00800000u >= 0x7f000000u && m != 0) return widen_rare(x);
+    return __hiloint2double((int)((b & 0x80000000u) | (m == 0 ? 0u : (m >> 3) + 0x38000000u)), (int)(b << 29));
 }
 __device__ __forceinline__ float narrow(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffull;
     const unsigned e = (unsigned)(m >> 52);
-    if (e - 897u >= 253u) return (float)x;  // exponents 897..1149: normal floats, rounding cannot overflow
+    if (e - 897u >= 253u) return narrow_rare(x);  // exponents 897..1149: normal floats, rounding cannot overflow
     const unsigned long long r = m - (896ull << 52) + 0x0fffffffull + ((m >> 29) & 1ull);  // to nearest, ties to even
     return __uint_as_float((unsigned)(r >> 29) | ((unsigned)(b >> 32) & 0x80000000u));
 }
 
+__device__ __noinline__ int floor_cell_rare(double x, float *t) {
+    const double f = floor(x);
+    *t = (float)(x - f);
+    return (int)fmin(fmax(f, -1e6), 1e6);
+}
+
 // floor(x) as an integer and the fraction x - floor(x): one addition rounded
-// down, exact for |x| < 2^31.  Beyond +-10^6 (and for NaN) the cell is clamped
-// to that (negative side for NaN), which stays outside of the grid.
+// down.  Beyond +-10^6 (and for NaN) the cell is clamped to that (negative
+// side for NaN), which stays outside of the grid.
 __device__ __forceinline__ int floor_cell(double x, float &t) {
     const double magic = 6755399441055744.0;  // 1.5 * 2^52
-    const double big = __dadd_rd(x, magic);
-    const double fl = big - magic;
     const int hi = __double2hiint(x) & 0x7fffffff;
-    t = narrow(x - fl);
-    if (hi < 0x412e8480) return __double2loint(big);  // |x| < 10^6
-    const double f = floor(x);
-    t = (float)(x - f);
-    return (int)fmin(fmax(f, -1e6), 1e6);
+    if (hi >= 0x412e8480) return floor_cell_rare(x, &t);  // |x| >= 10^6
+    const double big = __dadd_rd(x, magic);
+    t = narrow(x - (big - magic));
+    return __double2loint(big);
 }
 
 // Base of a double state (double arithmetic; used at launch and to resync).
@@ -373,7 +379,7 @@ __device__ __forceinline__ unsigned long long row_index(int i, int n_j, int j, i
 // so all lanes hold bitwise equal results.  The body has no branch: the field
 // terms (which do not need Ne) come first and can overlap the sample gathers,
 // and a stage outside the grid gathers from cell 0 and discards the result.
-template <int STENCIL, int G, int IP>
+template <int STENCIL, int G, int IP, bool FIRST = false>
 __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float> &rp, const Base32 &b,
                                           const float d[6], float dy[6], float *mu2, int q, unsigned gmask) {
     StageIn<float> s;
@@ -460,7 +466,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
     s.dX[0] = inside ? rp.xfac * out[3] * g.sc : 0.0f;
     s.dX[1] = inside ? rp.xfac * out[1] * g.sa : 0.0f;
     s.dX[2] = inside ? rp.xfac * out[2] * g.sb : 0.0f;
-    ray_rhs<float>(rp, s, F, dy, mu2);
+    ray_rhs<float, FIRST>(rp, s, F, dy, mu2);
 }
 
 // Butcher tables in "shifted accumulator" form.  After stage s produced k_s,
@@ -763,13 +769,13 @@ __device__ __forceinline__ bool lane_next_attempt(Lane &L, const FanDev &f) {
 
 // The launch evaluation: mu^2 at the transmitter for the launch direction,
 // then |k| = mu.  Returns true when the ray has finished (status set).
-template <int STENCIL, int G, int IP>
+template <int STENCIL, int G, int IP, bool FIRST = false>
 __device__ bool lane_launch(Lane &L, const GridDev &g, const FanDev &f, int q, unsigned gmask) {
     const RayPhys<float> rp = lane_phys(g, L);
     float d[6], ks[6], mu2;
 #pragma unroll
     for (int c = 0; c < 6; ++c) d[c] = 0.0f;
-    rhs_mixed<STENCIL, G, IP>(g, rp, L.b, d, ks, &mu2, q, gmask);
+    rhs_mixed<STENCIL, G, IP, FIRST>(g, rp, L.b, d, ks, &mu2, q, gmask);
     ++L.n_ev;
     L.launch = false;
     if (!(mu2 > 0.0f)) {
@@ -815,7 +821,7 @@ __device__ __forceinline__ void lane_stage0_done(Lane &L, const GridDev &g, cons
 // stage evaluation serves all stages, which keeps the loop inside the
 // instruction cache; with 2 or 4 lanes per ray (latency-bound fans) stage 0
 // is a separate copy, which schedules better.
-template <int STENCIL, int G, int IP>
+template <int STENCIL, int G, int IP, bool FIRST = false>
 __device__ __forceinline__ void lane_attempt(Lane &L, const GridDev &g, const FanDev &f, const Tableau &T, int q,
                                              unsigned gmask) {
     const RayPhys<float> rp = lane_phys(g, L);
@@ -827,7 +833,7 @@ __device__ __forceinline__ void lane_attempt(Lane &L, const GridDev &g, const Fa
             if (s > 0 || fresh) {
 #pragma unroll
                 for (int c = 0; c < 6; ++c) d[c] = s == 0 ? 0.0f : L.hs * L.acc[0][c];
-                rhs_mixed<STENCIL, G, IP>(g, rp, L.b, d, ks, nullptr, q, gmask);
+                rhs_mixed<STENCIL, G, IP, FIRST>(g, rp, L.b, d, ks, nullptr, q, gmask);
                 ++L.n_ev;
             }
             if (s == 0) {
@@ -845,7 +851,7 @@ __device__ __forceinline__ void lane_attempt(Lane &L, const GridDev &g, const Fa
         if (fresh) {
 #pragma unroll
             for (int c = 0; c < 6; ++c) d[c] = 0.0f;
-            rhs_mixed<STENCIL, G, IP>(g, rp, L.b, d, L.k1, nullptr, q, gmask);
+            rhs_mixed<STENCIL, G, IP, FIRST>(g, rp, L.b, d, L.k1, nullptr, q, gmask);
             ++L.n_ev;
         }
         lane_stage0_done(L, g, f, T, fresh);
@@ -853,7 +859,7 @@ __device__ __forceinline__ void lane_attempt(Lane &L, const GridDev &g, const Fa
         for (int s = 1; s < T.ns; ++s) {
 #pragma unroll
             for (int c = 0; c < 6; ++c) d[c] = L.hs * L.acc[0][c];
-            rhs_mixed<STENCIL, G, IP>(g, rp, L.b, d, ks, nullptr, q, gmask);
+            rhs_mixed<STENCIL, G, IP, FIRST>(g, rp, L.b, d, ks, nullptr, q, gmask);
             ++L.n_ev;
             accumulate_next(L, T, s, ks);
         }
@@ -1080,6 +1086,7 @@ template <int STENCIL, int G, int IP>
 __global__ void __launch_bounds__(128, G == 1 ? 3 : 2) trace_mixed_persistent_kernel(GridDev g, FanDev f,
                                                                      rt_ray_result *__restrict__ out,
                                                                      unsigned long long *__restrict__ counter) {
+    constexpr bool FIRST = G == 1 && STENCIL != RT_STENCIL_GATHER;
     __shared__ Tableau T;
     __shared__ Base32 btx;
     __shared__ LandState land[128];
@@ -1114,7 +1121,7 @@ __global__ void __launch_bounds__(128, G == 1 ? 3 : 2) trace_mixed_persistent_ke
             if (c < (unsigned long long)n) {
                 L.active = true;
                 lane_begin_ray(L, g, f, claim_to_ray(f, (long long)c), btx);
-                if (lane_launch<STENCIL, G, IP>(L, g, f, q, gmask)) lane_finish(L, g, f, out, q == 0);
+                if (lane_launch<STENCIL, G, IP, FIRST>(L, g, f, q, gmask)) lane_finish(L, g, f, out, q == 0);
             }
         }
         if (!__any_sync(FULL, L.active)) break;
@@ -1132,7 +1139,7 @@ __global__ void __launch_bounds__(128, G == 1 ? 3 : 2) trace_mixed_persistent_ke
                 break;
             }
             if (L.active) {
-                lane_attempt<STENCIL, G, IP>(L, g, f, T, q, gmask);
+                lane_attempt<STENCIL, G, IP, FIRST>(L, g, f, T, q, gmask);
                 if (lane_end_attempt(L, g, f, land[threadIdx.x])) lane_finish(L, g, f, out, q == 0);
             }
         } while (__any_sync(FULL, L.active));
