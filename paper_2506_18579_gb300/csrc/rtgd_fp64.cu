@@ -7,20 +7,23 @@
 // instructions are not: with one ray per lane an evaluation took ~770 FP64
 // warp instructions (23.8 us) however few rays the warp still held.
 //
-// Layout: a block is one warp that holds up to eight rays.  While n of them
-// are in flight, each is carried by a group of G = 32 / 2^ceil(log2 n) lanes,
+// Layout: a block's first warp holds up to eight rays.  While n of them are
+// in flight, each is carried by a group of G = 32 / 2^ceil(log2 n) lanes,
 // which share the evaluation's independent parts (the polynomials of the
 // weights, the 16 sample rows, the state components, the coordinates, the
 // divisions, the r/theta/phi components of the field and the ray equations):
-// ~250 FP64 instructions at G = 4, ~175 at G = 32 (7.7 us).  As rays end the
-// warp regroups, so that its last ray runs on all 32 lanes.  A ray's
-// arithmetic is the same operations in the same order for every G (only the
-// lane that performs them changes), so its record depends neither on G nor on
-// its warp mates.  Ray states live in shared memory (slots), so that
-// regrouping moves no data.  The host starts a warp with as many rays as fill
-// the GPU (fp64_rays_per_warp).  Measured, one thread per ray before / now:
-// 16 rays RK4 without a field 133 / 32 ms, one RKF45 ray 42.5 / 16.1 ms, 720
-// rays 189 / 69 ms, the 24,840-ray fan 418 / 174 ms.
+// ~250 FP64 instructions at G = 4, ~175 at G = 32.  As rays end the warp
+// regroups, so that its last ray runs on all 32 lanes; then the block's second
+// warp, which waited at a barrier, takes the ~40 of those 175 that need not
+// wait for the rest (Duo).  A ray's arithmetic is the same operations in the
+// same order for every G, with and without the second warp (only the lane that
+// performs them changes), so its record depends on neither nor on its warp
+// mates.  Ray states live in shared memory (slots), so that regrouping moves
+// no data.  The host starts a warp with as many rays as fill the GPU
+// (fp64_rays_per_warp).  Measured with one thread per ray / lane groups / and
+// the second warp: 16 rays RK4 without a field 133 / 32 / 24.6 ms, one RKF45
+// ray 42.5 / 16.1 / 11.9 ms (one evaluation 21.2 / 8.0 / 5.9 us), 522 rays
+// 85 / 19.3 / 16.7 ms, the 24,840-ray fan 418 / 172 / 157 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -182,23 +185,77 @@ __device__ __forceinline__ double face_axis64(double x, double v, int n) {
     return ok ? d : HUGE_VAL;
 }
 
+// Two warps on one ray.  A lone warp issues one FP64 instruction per 64 cycles,
+// four warps of an SM about 3.4, so a block has a second warp that takes
+// independent parts of an evaluation once the first warp's rays have come down
+// to one (until then it waits at a barrier).  Producer / consumer pairs of
+// named barriers: one warp signals (arrives), the other waits.
+struct Duo {
+    enum { kStart = 1, kDensity = 2, kField = 3, kGradients = 4 };  // barrier numbers (0 is __syncthreads)
+    enum { dXfac = 0, dM = 1, dA = 4, dA2, dYY, dKY, dIr, dIkk, dSth, dCth, dGYY, dGKY = dGYY + 3, dKV = dGKY + 3,
+           dKYn = dKV + 3, dC2, dSize };
+    double *D;          // shared: what the warps hand over
+    int *request;       // shared: offset of the stage state in the block's shared memory, -1 to stop
+    const double *sm;   // shared memory of the block
+
+    static __device__ __forceinline__ void signal(int barrier) {
+        __syncwarp();
+        __threadfence_block();
+        asm volatile("bar.arrive %0, 64;" ::"r"(barrier) : "memory");
+    }
+    static __device__ __forceinline__ void wait(int barrier) {
+        __syncwarp();
+        asm volatile("bar.sync %0, 64;" ::"r"(barrier) : "memory");
+    }
+    __device__ __forceinline__ void start(const double *ys, int lane) {
+        if (lane == 0) *(volatile int *)request = (int)(ys - sm);
+        signal(kStart);
+    }
+    __device__ __forceinline__ void stop(int lane) {
+        if (lane == 0) *(volatile int *)request = -1;
+        signal(kStart);
+    }
+};
+
+// Component j of the gradients of |Y|^2 and of k . Y (at fixed k):
+// gYY: (-6 YY) ir, ((6 A2) mr) mt, ((6 A2) mr) smp;
+// gkY: (-3 kY) ir, A ((-2 kr) mt - kt mr), A ((-2 kr) smp + (kt cth) mp - kp (sth mr + cth mt)).
+__device__ __forceinline__ void field_gradients(int j, double kr, double kt, double kp, double mr, double mt, double mj,
+                                                double A, double A2, double YY, double kY, double ir, double sth,
+                                                double cth, double &gYY, double &gkY) {
+    const double smp = __dmul_rn(sth, mj);  // j = 2
+    gYY = __dmul_rn(__dmul_rn(__dmul_rn(j == 0 ? -6.0 : 6.0, j == 0 ? YY : A2), j == 0 ? ir : mr),
+                    j == 0 ? 1.0 : j == 1 ? mt : smp);
+    const double m2kr = __dmul_rn(-2.0, kr), ktc = __dmul_rn(kt, cth);
+    const double inner = fma(sth, mr, __dmul_rn(cth, mt));
+    double e = __dmul_rn(j == 0 ? -3.0 : j == 1 ? -kt : ktc, j == 0 ? kY : j == 1 ? mr : mj);
+    e = fma(j == 0 ? 1.0 : m2kr, j == 0 ? -0.0 : j == 1 ? mt : smp, e);
+    e = fma(j < 2 ? 1.0 : -kp, j < 2 ? -0.0 : inner, e);
+    gkY = __dmul_rn(j == 0 ? ir : A, e);
+}
+
 // tail64 by a quad of lanes: lane j = 0, 1, 2 carries the r, theta, phi
 // component (lane 3 repeats lane 2), and the independent quotients and the
 // partials FX, FL, FT of Appleton-Hartree stand side by side in lanes 0-2.
 // The same operations in the same order as tail64 (a lane that has nothing to
 // do in a shared instruction multiplies by 1 or adds -0, which changes
 // nothing): ~110 FP64 instructions instead of ~175, without a field ~30
-// instead of ~45.  d and dk receive dy[j] and dy[3 + j]; dXj is s.dX[j].
-__device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const StageIn<double> &s, double dXj, int j,
-                                            double &d, double &dk) {
+// instead of ~45.  d and dk receive dy[j] and dy[3 + j].  X and its derivatives
+// are in C[cO ..] (see density64); DUO: the second warp forms them, and the
+// gradients of the field, meanwhile.
+template <bool DUO>
+__device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const StageIn<double> &s, const double *C, int j,
+                                            int q, Duo &duo, double &d, double &dk) {
     auto from = [](double v, int lane) { return __shfl_sync(kFull, v, lane, 4); };
-    const double kr = s.k[0], kt = s.k[1], kp = s.k[2], X = s.X;
+    const double kr = s.k[0], kt = s.k[1], kp = s.k[2];
     const double kj = j == 0 ? kr : j == 1 ? kt : kp;
     const double kk = fma(kp, kp, fma(kr, kr, __dmul_rn(kt, kt)));
     const double rc = __drcp_rn(j == 0 ? s.r : j == 1 ? s.sth : kk);
     const double ir = from(rc, 0), ist = from(rc, 1);
-    double H, K, G;
+    double H, K, G, kv = 0.0;
     if (rp.iso) {
+        if (DUO) Duo::wait(Duo::kDensity);
+        const double X = C[cO], dXj = C[cO + (j == 0 ? 3 : j)];
         H = __dmul_rn(0.5, dXj);
         K = kj;
         G = __dadd_rn(-kk, -X);
@@ -209,27 +266,35 @@ __device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const Sta
         const double px = __dmul_rn(rp.m[0], sj), py = __dmul_rn(rp.m[1], sj);
         const double mj = fma(j == 0 ? rp.m[2] : j == 1 ? -rp.m[2] : 1.0, j == 0 ? s.cth : j == 1 ? s.sth : -0.0,
                               fma(py, j < 2 ? s.sph : s.cph, __dmul_rn(px, j < 2 ? s.cph : -s.sph)));
-        const double q = __dmul_rn(rp.R_E, ir);
-        const double A = __dmul_rn(__dmul_rn(__dmul_rn(rp.ab0, q), q), q);
+        const double rr = __dmul_rn(rp.R_E, ir);
+        const double A = __dmul_rn(__dmul_rn(__dmul_rn(rp.ab0, rr), rr), rr);
         const double A2 = __dmul_rn(A, A);
         const double Yj = __dmul_rn(__dmul_rn(j == 0 ? -2.0 : 1.0, A), mj);
         const double mr = from(mj, 0), mt = from(mj, 1);
         const double kY = fma(kp, from(Yj, 2), fma(kr, from(Yj, 0), __dmul_rn(kt, from(Yj, 1))));
         const double YY = __dmul_rn(A2, fma(__dmul_rn(3.0, mr), mr, 1.0));
-        const double smp = __dmul_rn(s.sth, mj);  // lanes 2, 3
-        // gYY: (-6 YY) ir, ((6 A2) mr) mt, ((6 A2) mr) smp
-        const double gYY = __dmul_rn(__dmul_rn(__dmul_rn(j == 0 ? -6.0 : 6.0, j == 0 ? YY : A2), j == 0 ? ir : mr),
-                                     j == 0 ? 1.0 : j == 1 ? mt : smp);
-        // gkY: (-3 kY) ir, A ((-2 kr) mt - kt mr), A ((-2 kr) smp + (kt cth) mp - kp (sth mr + cth mt))
-        const double m2kr = __dmul_rn(-2.0, kr), ktc = __dmul_rn(kt, s.cth);
-        const double inner = fma(s.sth, mr, __dmul_rn(s.cth, mt));
-        double e = __dmul_rn(j == 0 ? -3.0 : j == 1 ? -kt : ktc, j == 0 ? kY : j == 1 ? mr : mj);
-        e = fma(j == 0 ? 1.0 : m2kr, j == 0 ? -0.0 : j == 1 ? mt : smp, e);
-        e = fma(j < 2 ? 1.0 : -kp, j < 2 ? -0.0 : inner, e);
-        const double gkY = __dmul_rn(j == 0 ? ir : A, e);
+        double gYY, gkY;
+        if (DUO) {
+            if (q < 3) duo.D[Duo::dM + q] = mj;
+            if (q == 0) {
+                duo.D[Duo::dA] = A;
+                duo.D[Duo::dA2] = A2;
+                duo.D[Duo::dYY] = YY;
+                duo.D[Duo::dKY] = kY;
+                duo.D[Duo::dIr] = ir;
+                duo.D[Duo::dIkk] = ikk;
+                duo.D[Duo::dSth] = s.sth;
+                duo.D[Duo::dCth] = s.cth;
+            }
+            Duo::signal(Duo::kField);
+        } else {
+            field_gradients(j, kr, kt, kp, mr, mt, mj, A, A2, YY, kY, ir, s.sth, s.cth, gYY, gkY);
+        }
         const double L = __dmul_rn(__dmul_rn(kY, kY), ikk);
         double T = __dadd_rn(YY, -L);
         if (T < 0.0) T = 0.0;
+        if (DUO) Duo::wait(Duo::kDensity);
+        const double X = C[cO], dXj = C[cO + (j == 0 ? 3 : j)];
         const double u = __dadd_rn(1.0, -X);
         const double L4u = __dmul_rn(__dmul_rn(4.0, L), u), L4uu = __dmul_rn(L4u, u);
         const double S = sqrt(fma(T, T, L4uu));
@@ -272,8 +337,19 @@ __device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const Sta
             F = __dmul_rn(fma(N, t, j == 0 ? -cD : -0.0), __dmul_rn(i1, i1));
         }
         const double FX = from(F, 0), FL = from(F, 1), FT = from(F, 2);
-        const double kYn = __dmul_rn(kY, ikk);
-        const double cL = __dmul_rn(__dadd_rn(FL, -FT), __dmul_rn(__dmul_rn(2.0, kY), ikk));
+        double kYn, c2;
+        if (DUO) {
+            Duo::wait(Duo::kGradients);
+            gYY = duo.D[Duo::dGYY + j];
+            gkY = duo.D[Duo::dGKY + j];
+            kv = duo.D[Duo::dKV + j];
+            kYn = duo.D[Duo::dKYn];
+            c2 = duo.D[Duo::dC2];
+        } else {
+            kYn = __dmul_rn(kY, ikk);
+            c2 = __dmul_rn(__dmul_rn(2.0, kY), ikk);
+        }
+        const double cL = __dmul_rn(__dadd_rn(FL, -FT), c2);
         const double hf = __dmul_rn(0.5, cL);
         H = __dmul_rn(-0.5, fma(cL, gkY, fma(FX, dXj, __dmul_rn(FT, gYY))));
         K = fma(-hf, fma(-kYn, kj, Yj), kj);
@@ -284,123 +360,175 @@ __device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const Sta
     d = __dmul_rn(__dmul_rn(-K, iG), sc);
     const double dr = from(d, 0), dt = from(d, 1), dp = from(d, 2);
     // kp sth in lane 0, (kp r) cth in lanes 1, 2
-    const double kv = __dmul_rn(__dmul_rn(kp, j == 0 ? s.sth : s.r), j == 0 ? 1.0 : s.cth);
+    if (!DUO || rp.iso) kv = __dmul_rn(__dmul_rn(kp, j == 0 ? s.sth : s.r), j == 0 ? 1.0 : s.cth);
     const double kps = from(kv, 0);
     double t = __dmul_rn(j == 0 ? kt : j == 1 ? -kt : -kps, j == 0 ? dt : dr);
     t = fma(j < 2 ? kv : -kv, j < 2 ? dp : dt, fma(H, iG, t));
     dk = __dmul_rn(t, sc);
 }
 
-// dy/dP' at the stage state yt by the G lanes of a group (lane q, scratch C),
-// into out (6 doubles of shared memory) if write is set; coef: the weight
-// polynomials of the grid's interpolant; returns sin(theta).  Called by whole
-// warps only (it holds barriers and shuffles).
+// X and its derivatives along r, theta, phi at the stage state ys by the G
+// lanes of a group (lane q): into C[cO .. cO + 3] as X, dX/dtheta, dX/dphi,
+// dX/dr, zeros outside the grid.  coef: the weight polynomials of the grid's
+// interpolant.  Called by whole warps only (it holds barriers); the caller
+// synchronises the warp before reading the result.
 template <int G>
-__device__ __forceinline__ double stage64(const GridDev &g, const RayPhys<double> &rp, const double yt[6], double *C,
-                                          const double *coef, int q, double *out, bool write) {
-    static_assert(G >= 4, "an axis and a component per lane of a quad");
-    StageIn<double> s;
-    s.r = yt[0];
-    s.k[0] = yt[3];
-    s.k[1] = yt[4];
-    s.k[2] = yt[5];
+__device__ __forceinline__ void density64(const GridDev &g, double xfac, const double *ys, double *C,
+                                          const double *coef, int q) {
+    static_assert(G >= 4, "an axis per lane");
     // cells: an axis per lane
     int *cell = (int *)(C + cCell);
     if (q < 3) {
         int i;
         double t;
-        const bool ok = cell64(grid_coord64(g, q, yt[0], yt[1], yt[2]), q == 0 ? g.n_lat : q == 1 ? g.n_lon : g.n_alt, i, t);
+        const bool ok = cell64(grid_coord64(g, q, ys[0], ys[1], ys[2]), q == 0 ? g.n_lat : q == 1 ? g.n_lon : g.n_alt, i, t);
         C[cFrac + q] = t;
         cell[q] = ok ? i : -1;
     }
-    // sines and cosines: theta on the even lanes, phi on the odd ones
+    __syncwarp();
+    const int ca = cell[0], cb = cell[1], cc = cell[2];
+    const bool inside = (ca | cb | cc) >= 0;
+    if (!__any_sync(kFull, inside)) {
+        if (q < 4) C[cO + q] = 0.0;
+        return;
+    }
+    // the 24 weights: weight p = 8 axis + 4 derivative + node, one polynomial each
+    for (int p = q; p < 24; p += G) {
+        const int node = p & 3, der = (p >> 2) & 1;
+        const bool right = node >= 2;
+        const bool outer = node == 0 || node == 3;  // nodes j-1, j+2
+        const double *cf = coef + (der * 2 + (outer ? 0 : 1)) * 5;
+        double t = C[cFrac + (p >> 3)];
+        t = right ? 1.0 - t : t;
+        double w = fma(t, cf[0], cf[1]);
+        w = fma(t, w, cf[2]);
+        w = fma(t, w, cf[3]);
+        // kinds 0, 2: one more Horner step; kind 1: t^2; kind 3: times t (adding -0 changes nothing)
+        const double w4 = fma(t, (der | (int)outer) ? w : t, outer ? cf[4] : -0.0);
+        const double w5 = __dmul_rn(w4, outer ? t : w);
+        w = der ? w4 : __dadd_rn(outer ? -0.0 : 1.0, w5);
+        C[cW + p] = (der && right) ? -w : w;
+    }
+    __syncwarp();
+    const long long sj = g.p_alt, si = (long long)g.p_lon * g.p_alt;
+    const double *base = g.pad64 + (long long)(inside ? ca : 0) * si + (long long)(inside ? cb : 0) * sj + (inside ? cc : 0);
+    // altitude rows (Eq. 13): row 4 a + b; with 32 lanes the upper half forms the derivative sums
+    if (G == 32) {
+        const int row = q & 15;
+        const double *p = base + (row >> 2) * si + (row & 3) * sj;
+        const double *w = C + cW + 16 + ((q >> 4) << 2);
+        C[cV + q] = fma(__ldg(p + 3), w[3], fma(__ldg(p + 2), w[2], fma(__ldg(p), w[0], __dmul_rn(__ldg(p + 1), w[1]))));
+    } else {
+        for (int row = q; row < 16; row += G) {
+            const double *p = base + (row >> 2) * si + (row & 3) * sj;
+            double v, dv;
+            row4<double>(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3), C + cW + 16, C + cW + 20, v, dv);
+            C[cV + row] = v;
+            C[cV + 16 + row] = dv;
+        }
+    }
+    __syncwarp();
+    // longitude: for each a the sums of v wb, v db, dv wb
+    for (int id = q; id < 12; id += G) {
+        const int a = id / 3, j = id - 3 * a;
+        const double *v = C + cV + (j == 2 ? 16 : 0) + 4 * a;
+        const double *w = C + cW + 8 + (j == 1 ? 4 : 0);
+        double sum = 0.0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) sum += v[b] * w[b];
+        C[cS + id] = sum;
+    }
+    __syncwarp();
+    // latitude, then to X and its derivatives
+    for (int o = q; o < 4; o += G) {
+        const double *v = C + cS + (o == 3 ? 2 : o == 2 ? 1 : 0);
+        const double *w = C + cW + (o == 1 ? 4 : 0);
+        double sum = 0.0;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) sum += v[3 * a] * w[a];
+        const double c1 = o == 0 ? 1.0 : o == 1 ? g.inv_dlat : o == 2 ? g.inv_dlon : g.inv_dalt;
+        const double c2 = o == 1 || o == 2 ? kRad2Deg : 1.0;
+        C[cO + o] = inside ? (o == 1 ? -xfac : xfac) * sum * c1 * c2 : 0.0;
+    }
+}
+
+// The warp's rays' sines and cosines: theta on the even lanes, phi on the odd ones.
+__device__ __forceinline__ void angles64(StageIn<double> &s, const double *ys, int q) {
+    s.r = ys[0];
+    s.k[0] = ys[3];
+    s.k[1] = ys[4];
+    s.k[2] = ys[5];
     double sn, cs;
-    sincos((q & 1) ? yt[2] : yt[1], &sn, &cs);
+    sincos(ys[1 + (q & 1)], &sn, &cs);
     const double so = __shfl_xor_sync(kFull, sn, 1), co = __shfl_xor_sync(kFull, cs, 1);
     s.sth = (q & 1) ? so : sn;
     s.cth = (q & 1) ? co : cs;
     s.sph = (q & 1) ? sn : so;
     s.cph = (q & 1) ? cs : co;
-    __syncwarp();
-    const int ca = cell[0], cb = cell[1], cc = cell[2];
-    const bool inside = (ca | cb | cc) >= 0;
+}
+
+// dy/dP' at the stage state ys (6 doubles of shared memory) by the G lanes of
+// a group (lane q, scratch C), into out if write is set; returns sin(theta).
+// Called by whole warps only.  With 32 lanes the block's second warp helps
+// (Duo): it forms X and its derivatives while this one forms the sines, the
+// field and Appleton-Hartree's arguments, and the field's gradients while this
+// one goes through Appleton-Hartree.
+template <int G>
+__device__ __forceinline__ double stage64(const GridDev &g, const RayPhys<double> &rp, const double *ys, double *C,
+                                          const double *coef, int q, double *out, bool write, Duo &duo) {
+    StageIn<double> s;
     const int j = (q & 3) == 3 ? 2 : (q & 3);  // the component this lane carries
-    double dXj = 0.0;
-    s.X = 0.0;
-    if (__any_sync(kFull, inside)) {
-        // the 24 weights: weight p = 8 axis + 4 derivative + node, one polynomial each
-        for (int p = q; p < 24; p += G) {
-            const int node = p & 3, der = (p >> 2) & 1;
-            const bool right = node >= 2;
-            const bool outer = node == 0 || node == 3;  // nodes j-1, j+2
-            const double *cf = coef + (der * 2 + (outer ? 0 : 1)) * 5;
-            double t = C[cFrac + (p >> 3)];
-            t = right ? 1.0 - t : t;
-            double w = fma(t, cf[0], cf[1]);
-            w = fma(t, w, cf[2]);
-            w = fma(t, w, cf[3]);
-            // kinds 0, 2: one more Horner step; kind 1: t^2; kind 3: times t (adding -0 changes nothing)
-            const double w4 = fma(t, (der | (int)outer) ? w : t, outer ? cf[4] : -0.0);
-            const double w5 = __dmul_rn(w4, outer ? t : w);
-            w = der ? w4 : __dadd_rn(outer ? -0.0 : 1.0, w5);
-            C[cW + p] = (der && right) ? -w : w;
-        }
-        __syncwarp();
-        const long long sj = g.p_alt, si = (long long)g.p_lon * g.p_alt;
-        const double *base = g.pad64 + (long long)(inside ? ca : 0) * si + (long long)(inside ? cb : 0) * sj +
-                             (inside ? cc : 0);
-        // altitude rows (Eq. 13): row 4 a + b; with 32 lanes the upper half forms the derivative sums
-        if (G == 32) {
-            const int row = q & 15;
-            const double *p = base + (row >> 2) * si + (row & 3) * sj;
-            const double *w = C + cW + 16 + ((q >> 4) << 2);
-            C[cV + q] = fma(__ldg(p + 3), w[3], fma(__ldg(p + 2), w[2], fma(__ldg(p), w[0], __dmul_rn(__ldg(p + 1), w[1]))));
-        } else {
-            for (int row = q; row < 16; row += G) {
-                const double *p = base + (row >> 2) * si + (row & 3) * sj;
-                double v, dv;
-                row4<double>(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3), C + cW + 16, C + cW + 20, v, dv);
-                C[cV + row] = v;
-                C[cV + 16 + row] = dv;
-            }
-        }
-        __syncwarp();
-        // longitude: for each a the sums of v wb, v db, dv wb
-        for (int id = q; id < 12; id += G) {
-            const int a = id / 3, j = id - 3 * a;
-            const double *v = C + cV + (j == 2 ? 16 : 0) + 4 * a;
-            const double *w = C + cW + 8 + (j == 1 ? 4 : 0);
-            double sum = 0.0;
-#pragma unroll
-            for (int b = 0; b < 4; ++b) sum += v[b] * w[b];
-            C[cS + id] = sum;
-        }
-        __syncwarp();
-        // latitude, then to X and its derivatives along r, theta, phi: lane o
-        // forms X (0), dX/dtheta (1), dX/dphi (2), dX/dr (3)
-        for (int o = q; o < 4; o += G) {
-            const double *v = C + cS + (o == 3 ? 2 : o == 2 ? 1 : 0);
-            const double *w = C + cW + (o == 1 ? 4 : 0);
-            double sum = 0.0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) sum += v[3 * a] * w[a];
-            const double c1 = o == 0 ? 1.0 : o == 1 ? g.inv_dlat : o == 2 ? g.inv_dlon : g.inv_dalt;
-            const double c2 = o == 1 || o == 2 ? kRad2Deg : 1.0;
-            C[cO + o] = (o == 1 ? -rp.xfac : rp.xfac) * sum * c1 * c2;
-        }
-        __syncwarp();
-        if (inside) {
-            s.X = C[cO];
-            dXj = C[cO + (j == 0 ? 3 : j)];
-        }
-    }
     double d, dk;
-    tail64_quad(rp, s, dXj, j, d, dk);
+    if (G == 32) {
+        duo.start(ys, q);
+        angles64(s, ys, q);
+        tail64_quad<true>(rp, s, C, j, q, duo, d, dk);
+    } else {
+        density64<G>(g, rp.xfac, ys, C, coef, q);
+        angles64(s, ys, q);
+        __syncwarp();
+        tail64_quad<false>(rp, s, C, j, q, duo, d, dk);
+    }
     if (write && q < 3) {
         out[q] = d;
         out[3 + q] = dk;
     }
     return s.sth;
+}
+
+// The second warp of a block: serves the first one's requests until it is
+// told to stop.  The requests' sequence is fixed (start, density, and with a
+// field the gradients), so every barrier's two sides always meet.
+__device__ __forceinline__ void helper64(const GridDev &g, const double *sm, double *C, const double *coef, int lane,
+                                         Duo &duo) {
+    const int j = (lane & 3) == 3 ? 2 : (lane & 3);
+    for (;;) {
+        Duo::wait(Duo::kStart);
+        const int at = *(volatile int *)duo.request;
+        if (at < 0) return;
+        const double *ys = sm + at;
+        density64<32>(g, duo.D[Duo::dXfac], ys, C, coef, lane);
+        Duo::signal(Duo::kDensity);
+        if (g.iso != 0) continue;
+        Duo::wait(Duo::kField);
+        const double *D = duo.D;
+        const double kr = ys[3], kt = ys[4], kp = ys[5];
+        const double mr = D[Duo::dM], mt = D[Duo::dM + 1], mj = D[Duo::dM + j], A = D[Duo::dA], kY = D[Duo::dKY];
+        const double ir = D[Duo::dIr], sth = D[Duo::dSth], cth = D[Duo::dCth], ikk = D[Duo::dIkk];
+        double gYY, gkY;
+        field_gradients(j, kr, kt, kp, mr, mt, mj, A, D[Duo::dA2], D[Duo::dYY], kY, ir, sth, cth, gYY, gkY);
+        if (lane < 3) {
+            duo.D[Duo::dGYY + lane] = gYY;
+            duo.D[Duo::dGKY + lane] = gkY;
+            duo.D[Duo::dKV + lane] = __dmul_rn(__dmul_rn(kp, j == 0 ? sth : ys[0]), j == 0 ? 1.0 : cth);
+        }
+        const double kYn = __dmul_rn(kY, ikk), c2 = __dmul_rn(__dmul_rn(2.0, kY), ikk);
+        if (lane == 0) {
+            duo.D[Duo::dKYn] = kYn;
+            duo.D[Duo::dC2] = c2;
+        }
+        Duo::signal(Duo::kGradients);
+    }
 }
 
 // Raw final state of a ray into its record (the angles stand in the
@@ -432,8 +560,8 @@ __device__ __forceinline__ void write_raw(rt_ray_result *out, int id, double P, 
 template <int G>
 __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, double *slots, double *scratch,
                                          const double *coef, const double *pow2q, int *map, int &n_act,
-                                         rt_ray_result *__restrict__ out) {
-    const int lane = threadIdx.x, grp = lane / G, q = lane % G;
+                                         rt_ray_result *__restrict__ out, Duo &duo) {
+    const int lane = threadIdx.x, grp = lane / G, q = lane % G;  // the block's first warp
     const bool has = grp < n_act;
     const int slot = map[has ? grp : 0];
     double *S = slots + slot * kSlot;
@@ -457,6 +585,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
     const int id = SI[kId];
     bool live = has;
     const bool writer = q == 0;
+    if (G == 32 && writer) duo.D[Duo::dXfac] = rp.xfac;
     __syncwarp();
     for (;;) {
         const unsigned am = __ballot_sync(kFull, live && writer);
@@ -481,13 +610,10 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
             if (writer) write_raw(out, id, P, S[kY + 1], S[kY + 2], apo, RT_RAY_MAX_STEPS, steps, att, ev);
             live = false;
         }
-        double yt[6];
         // k1 where it is not known (a new state)
         const bool need = live && !(flags & kK1Valid);
         if (__any_sync(kFull, need)) {
-#pragma unroll
-            for (int i = 0; i < 6; ++i) yt[i] = S[kY + i];
-            const double sth = stage64<G>(g, rp, yt, C, coef, q, S + kK1, need);
+            const double sth = stage64<G>(g, rp, S + kY, C, coef, q, S + kK1, need, duo);
             if (need) {
                 ++ev;
                 flags |= kK1Valid;
@@ -533,9 +659,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
                                      : fma(s == 3 ? hs : 0.5 * hs, s == 1 ? S[kK1 + c] : C[cK + 6 * (s - 2) + c], y);
             }
             __syncwarp();
-#pragma unroll
-            for (int i = 0; i < 6; ++i) yt[i] = C[cT + i];
-            stage64<G>(g, rp, yt, C, coef, q, C + cK + 6 * (s - 1), true);
+            stage64<G>(g, rp, C + cT, C, coef, q, C + cK + 6 * (s - 1), true, duo);
             __syncwarp();
         }
         if (adaptive) {
@@ -666,19 +790,25 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
 
 // Bytes of shared memory of a block that starts with R rays.
 constexpr size_t fp64_smem_bytes(int R) {
-    return sizeof(double) * (size_t)(kPoly + kPow2 + R * (kSlot + cGroup)) + kMaxRays * sizeof(int);
+    return sizeof(double) * (size_t)(kPoly + kPow2 + Duo::dSize + R * (kSlot + cGroup)) + (kMaxRays + 1) * sizeof(int);
 }
 static_assert(fp64_smem_bytes(kMaxRays) <= 48 * 1024, "fits the default shared-memory limit");
 
-// One warp per block; R rays (a power of two, at most kMaxRays) per warp at
-// the start.
-__global__ void __launch_bounds__(32) trace_fp64_kernel(const __grid_constant__ GridDev g,
+// A warp with R rays (a power of two, at most kMaxRays) at the start and its
+// helper per block.
+__global__ void __launch_bounds__(64) trace_fp64_kernel(const __grid_constant__ GridDev g,
                                                         const __grid_constant__ FanDev f, int R,
                                                         rt_ray_result *__restrict__ out) {
     extern __shared__ double sm[];
-    double *coef = sm, *pow2q = coef + kPoly, *slots = pow2q + kPow2, *scratch = slots + R * kSlot;
+    double *coef = sm, *pow2q = coef + kPoly, *hand = pow2q + kPow2, *slots = hand + Duo::dSize,
+           *scratch = slots + R * kSlot;
     int *map = (int *)(scratch + R * cGroup);
-    const int lane = threadIdx.x;
+    Duo duo{hand, map + kMaxRays, sm};
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x >= 32) {
+        helper64(g, sm, scratch, coef, lane, duo);
+        return;
+    }
     if (lane < kPoly) coef[lane] = (&c_poly[g.interp == 1 ? 1 : 0][0][0])[lane];
     if (lane < kPow2) pow2q[lane] = exp2((double)(lane - 10) * 0.25);
     // launch: |k| = mu at the transmitter (one ray per lane; spare lanes do nothing)
@@ -721,11 +851,12 @@ __global__ void __launch_bounds__(32) trace_fp64_kernel(const __grid_constant__ 
     __syncwarp();
     int n_act = __popc(am);
     while (n_act > 0) {
-        if (n_act > 4) run_rays<4>(g, f, slots, scratch, coef, pow2q, map, n_act, out);
-        else if (n_act > 2) run_rays<8>(g, f, slots, scratch, coef, pow2q, map, n_act, out);
-        else if (n_act > 1) run_rays<16>(g, f, slots, scratch, coef, pow2q, map, n_act, out);
-        else run_rays<32>(g, f, slots, scratch, coef, pow2q, map, n_act, out);
+        if (n_act > 4) run_rays<4>(g, f, slots, scratch, coef, pow2q, map, n_act, out, duo);
+        else if (n_act > 2) run_rays<8>(g, f, slots, scratch, coef, pow2q, map, n_act, out, duo);
+        else if (n_act > 1) run_rays<16>(g, f, slots, scratch, coef, pow2q, map, n_act, out, duo);
+        else run_rays<32>(g, f, slots, scratch, coef, pow2q, map, n_act, out, duo);
     }
+    duo.stop(lane);
 }
 
 }  // namespace
@@ -734,10 +865,11 @@ __global__ void __launch_bounds__(32) trace_fp64_kernel(const __grid_constant__ 
 // its SM holds fewer than ~3.4 warps and 19 cycles per resident warp above
 // that; kCost is what an evaluation takes in FP64 instructions at 4, 8, 16 and
 // 32 lanes per ray.  The size with the least product is taken.  Measured at 8 /
-// 4 / 2 / 1 rays per warp: 16 rays 54 / 43 / 36 / 32 ms, 522 rays 27 / 23 / 21 /
-// 19 ms, 3,232 rays 49 / 46 / 70 / 99 ms, 4,968 rays 135 / 142 / 146 / 173 ms,
-// 24,840 rays 174 / 223 / 352 ms / -.  More rays per warp (one or two lanes
-// each) were no faster at any size: 24,840 rays 184 ms with 32, 177 with 16.
+// 4 / 2 / 1 rays per warp: 16 rays 54 / 42 / 36 / 25 ms, 522 rays 27 / 22 / 20 /
+// 17 ms, 3,232 rays 45 / 43 / 61 / 95 ms, 4,968 rays 106 / 108 / 113 / 152 ms,
+// 24,840 rays 157 / 214 / 341 ms / -.  More rays per warp (one or two lanes
+// each) were no faster at any size: 24,840 rays 184 ms with 32, 177 with 16,
+// against 174 with 8, all before the second warp.
 int fp64_rays_per_warp(long long n_rays, int sms) {
     static const double kCost[4] = {226, 205, 190, 175};
     double best = 1e300;
@@ -758,7 +890,7 @@ cudaError_t launch_trace_fp64(const GridDev &g, const FanDev &f, int rays_per_wa
                               cudaStream_t st) {
     const int R = rays_per_warp;
     const long long blocks = (f.n_rays + R - 1) / R;
-    trace_fp64_kernel<<<(unsigned)blocks, 32, fp64_smem_bytes(R), st>>>(g, f, R, out);
+    trace_fp64_kernel<<<(unsigned)blocks, 64, fp64_smem_bytes(R), st>>>(g, f, R, out);
     return cudaGetLastError();
 }
 
