@@ -13,17 +13,19 @@
 // weights, the 16 sample rows, the state components, the coordinates, the
 // divisions, the r/theta/phi components of the field and the ray equations):
 // ~250 FP64 instructions at G = 4, ~175 at G = 32.  As rays end the warp
-// regroups, so that its last ray runs on all 32 lanes; then the block's second
-// warp, which waited at a barrier, takes the ~40 of those 175 that need not
-// wait for the rest (Duo).  A ray's arithmetic is the same operations in the
-// same order for every G, with and without the second warp (only the lane that
-// performs them changes), so its record depends on neither nor on its warp
+// regroups, so that its last ray runs on all 32 lanes.  The block's second
+// warp takes the part of an evaluation that need not wait for the rest (Duo):
+// the electron density, ~90 of the 250 instructions at G = 4, ~25 of the 175 at
+// G = 32 and there the field's gradients (~15) too.  A ray's arithmetic is the
+// same operations in the same order for every G (only the warp and lane that
+// perform them change), so its record depends neither on G nor on its warp
 // mates.  Ray states live in shared memory (slots), so that regrouping moves
 // no data.  The host starts a warp with as many rays as fill the GPU
 // (fp64_rays_per_warp).  Measured with one thread per ray / lane groups / and
-// the second warp: 16 rays RK4 without a field 133 / 32 / 24.6 ms, one RKF45
-// ray 42.5 / 16.1 / 11.9 ms (one evaluation 21.2 / 8.0 / 5.9 us), 522 rays
-// 85 / 19.3 / 16.7 ms, the 24,840-ray fan 418 / 172 / 157 ms.
+// the second warp: 16 rays RK4 without a field 133 / 32 / 24.9 ms, one RKF45
+// ray 42.5 / 16.1 / 11.9 ms (one evaluation 21.2 / 8.0 / 5.9 us), 522 rays - /
+// 19.3 / 16.6 ms, 3,232 rays - / 49.0 / 39.5 ms, the 24,840-ray fan 418 / 172 /
+// 149 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -187,16 +189,22 @@ __device__ __forceinline__ double face_axis64(double x, double v, int n) {
 
 // Two warps on one ray.  A lone warp issues one FP64 instruction per 64 cycles,
 // four warps of an SM about 3.4, so a block has a second warp that takes
-// independent parts of an evaluation once the first warp's rays have come down
-// to one (until then it waits at a barrier).  Producer / consumer pairs of
-// named barriers: one warp signals (arrives), the other waits.
+// independent parts of every evaluation: X and its derivatives for all of the
+// first warp's groups, and once a single ray is left (32 lanes) the gradients
+// of its field.  Producer / consumer pairs of named barriers: one warp signals
+// (arrives), the other waits.
 struct Duo {
     enum { kStart = 1, kDensity = 2, kField = 3, kGradients = 4 };  // barrier numbers (0 is __syncthreads)
     enum { dXfac = 0, dM = 1, dA = 4, dA2, dYY, dKY, dIr, dIkk, dSth, dCth, dGYY, dGKY = dGYY + 3, dKV = dGKY + 3,
            dKYn = dKV + 3, dC2, dSize };
     double *D;          // shared: what the warps hand over
-    int *request;       // shared: offset of the stage state in the block's shared memory, -1 to stop
-    const double *sm;   // shared memory of the block
+    // shared: lanes per ray G (+ kState: at the rays' states instead of their
+    // stage states), 0 to stop; for the single ray of G = 32 instead kSingle times
+    // 1 + the offset of its (stage) state in the block's shared memory
+    int *request;
+    int *slot_of;       // shared: the slot of each group's ray
+    const double *sm;   // the block's shared memory
+    enum { kState = 64, kSingle = 256 };
 
     static __device__ __forceinline__ void signal(int barrier) {
         __syncwarp();
@@ -207,12 +215,8 @@ struct Duo {
         __syncwarp();
         asm volatile("bar.sync %0, 64;" ::"r"(barrier) : "memory");
     }
-    __device__ __forceinline__ void start(const double *ys, int lane) {
-        if (lane == 0) *(volatile int *)request = (int)(ys - sm);
-        signal(kStart);
-    }
-    __device__ __forceinline__ void stop(int lane) {
-        if (lane == 0) *(volatile int *)request = -1;
+    __device__ __forceinline__ void start(int what, int lane) {
+        if (lane == 0) *(volatile int *)request = what;
         signal(kStart);
     }
 };
@@ -241,9 +245,9 @@ __device__ __forceinline__ void field_gradients(int j, double kr, double kt, dou
 // do in a shared instruction multiplies by 1 or adds -0, which changes
 // nothing): ~110 FP64 instructions instead of ~175, without a field ~30
 // instead of ~45.  d and dk receive dy[j] and dy[3 + j].  X and its derivatives
-// are in C[cO ..] (see density64); DUO: the second warp forms them, and the
-// gradients of the field, meanwhile.
-template <bool DUO>
+// come from the second warp in C[cO ..] (see density64); GRAD: so do the
+// gradients of the field.
+template <bool GRAD>
 __device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const StageIn<double> &s, const double *C, int j,
                                             int q, Duo &duo, double &d, double &dk) {
     auto from = [](double v, int lane) { return __shfl_sync(kFull, v, lane, 4); };
@@ -254,7 +258,7 @@ __device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const Sta
     const double ir = from(rc, 0), ist = from(rc, 1);
     double H, K, G, kv = 0.0;
     if (rp.iso) {
-        if (DUO) Duo::wait(Duo::kDensity);
+        Duo::wait(Duo::kDensity);
         const double X = C[cO], dXj = C[cO + (j == 0 ? 3 : j)];
         H = __dmul_rn(0.5, dXj);
         K = kj;
@@ -274,7 +278,7 @@ __device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const Sta
         const double kY = fma(kp, from(Yj, 2), fma(kr, from(Yj, 0), __dmul_rn(kt, from(Yj, 1))));
         const double YY = __dmul_rn(A2, fma(__dmul_rn(3.0, mr), mr, 1.0));
         double gYY, gkY;
-        if (DUO) {
+        if (GRAD) {
             if (q < 3) duo.D[Duo::dM + q] = mj;
             if (q == 0) {
                 duo.D[Duo::dA] = A;
@@ -293,7 +297,7 @@ __device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const Sta
         const double L = __dmul_rn(__dmul_rn(kY, kY), ikk);
         double T = __dadd_rn(YY, -L);
         if (T < 0.0) T = 0.0;
-        if (DUO) Duo::wait(Duo::kDensity);
+        Duo::wait(Duo::kDensity);
         const double X = C[cO], dXj = C[cO + (j == 0 ? 3 : j)];
         const double u = __dadd_rn(1.0, -X);
         const double L4u = __dmul_rn(__dmul_rn(4.0, L), u), L4uu = __dmul_rn(L4u, u);
@@ -338,7 +342,7 @@ __device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const Sta
         }
         const double FX = from(F, 0), FL = from(F, 1), FT = from(F, 2);
         double kYn, c2;
-        if (DUO) {
+        if (GRAD) {
             Duo::wait(Duo::kGradients);
             gYY = duo.D[Duo::dGYY + j];
             gkY = duo.D[Duo::dGKY + j];
@@ -360,7 +364,7 @@ __device__ __forceinline__ void tail64_quad(const RayPhys<double> &rp, const Sta
     d = __dmul_rn(__dmul_rn(-K, iG), sc);
     const double dr = from(d, 0), dt = from(d, 1), dp = from(d, 2);
     // kp sth in lane 0, (kp r) cth in lanes 1, 2
-    if (!DUO || rp.iso) kv = __dmul_rn(__dmul_rn(kp, j == 0 ? s.sth : s.r), j == 0 ? 1.0 : s.cth);
+    if (!GRAD || rp.iso) kv = __dmul_rn(__dmul_rn(kp, j == 0 ? s.sth : s.r), j == 0 ? 1.0 : s.cth);
     const double kps = from(kv, 0);
     double t = __dmul_rn(j == 0 ? kt : j == 1 ? -kt : -kps, j == 0 ? dt : dr);
     t = fma(j < 2 ? kv : -kv, j < 2 ? dp : dt, fma(H, iG, t));
@@ -467,28 +471,22 @@ __device__ __forceinline__ void angles64(StageIn<double> &s, const double *ys, i
     s.cph = (q & 1) ? cs : co;
 }
 
-// dy/dP' at the stage state ys (6 doubles of shared memory) by the G lanes of
-// a group (lane q, scratch C), into out if write is set; returns sin(theta).
-// Called by whole warps only.  With 32 lanes the block's second warp helps
-// (Duo): it forms X and its derivatives while this one forms the sines, the
-// field and Appleton-Hartree's arguments, and the field's gradients while this
-// one goes through Appleton-Hartree.
+// dy/dP' at the stage state ys (6 doubles of shared memory: the ray's state if
+// at_state, else C + cT) by the G lanes of a group (lane q, scratch C), into out
+// if write is set; returns sin(theta).  Called by the whole first warp only.
+// The block's second warp helps (Duo): it forms X and its derivatives while
+// this one forms the sines, the field and Appleton-Hartree's arguments, and
+// with 32 lanes the field's gradients while this one goes through
+// Appleton-Hartree.
 template <int G>
-__device__ __forceinline__ double stage64(const GridDev &g, const RayPhys<double> &rp, const double *ys, double *C,
-                                          const double *coef, int q, double *out, bool write, Duo &duo) {
+__device__ __forceinline__ double stage64(const RayPhys<double> &rp, const double *ys, bool at_state, const double *C,
+                                          int q, double *out, bool write, Duo &duo) {
     StageIn<double> s;
     const int j = (q & 3) == 3 ? 2 : (q & 3);  // the component this lane carries
     double d, dk;
-    if (G == 32) {
-        duo.start(ys, q);
-        angles64(s, ys, q);
-        tail64_quad<true>(rp, s, C, j, q, duo, d, dk);
-    } else {
-        density64<G>(g, rp.xfac, ys, C, coef, q);
-        angles64(s, ys, q);
-        __syncwarp();
-        tail64_quad<false>(rp, s, C, j, q, duo, d, dk);
-    }
+    duo.start(G == 32 ? Duo::kSingle * (1 + (int)(ys - duo.sm)) : G + (at_state ? Duo::kState : 0), threadIdx.x);
+    angles64(s, ys, q);
+    tail64_quad<G == 32>(rp, s, C, j, q, duo, d, dk);
     if (write && q < 3) {
         out[q] = d;
         out[3 + q] = dk;
@@ -496,18 +494,37 @@ __device__ __forceinline__ double stage64(const GridDev &g, const RayPhys<double
     return s.sth;
 }
 
+// X and its derivatives for every group of the first warp.
+template <int G>
+__device__ __forceinline__ void densities64(const GridDev &g, const double *slots, double *scratch, const double *coef,
+                                            int lane, bool at_state, const Duo &duo) {
+    const int grp = lane / G;
+    const double *S = slots + duo.slot_of[grp] * kSlot;
+    double *C = scratch + grp * cGroup;
+    density64<G>(g, S[kXfac], at_state ? S + kY : C + cT, C, coef, lane % G);
+}
+
 // The second warp of a block: serves the first one's requests until it is
-// told to stop.  The requests' sequence is fixed (start, density, and with a
-// field the gradients), so every barrier's two sides always meet.
-__device__ __forceinline__ void helper64(const GridDev &g, const double *sm, double *C, const double *coef, int lane,
-                                         Duo &duo) {
+// told to stop.  The requests' sequence is fixed (start, density, and for a
+// single ray in a field the gradients), so every barrier's two sides always meet.
+__device__ __forceinline__ void helper64(const GridDev &g, const double *slots, double *scratch, const double *coef,
+                                         int lane, Duo &duo) {
     const int j = (lane & 3) == 3 ? 2 : (lane & 3);
     for (;;) {
         Duo::wait(Duo::kStart);
-        const int at = *(volatile int *)duo.request;
-        if (at < 0) return;
-        const double *ys = sm + at;
-        density64<32>(g, duo.D[Duo::dXfac], ys, C, coef, lane);
+        const int what = *(volatile int *)duo.request;
+        if (what == 0) return;
+        if (what < Duo::kSingle) {  // the densities of several rays
+            const bool at_state = (what & Duo::kState) != 0;
+            const int G = what & (Duo::kState - 1);
+            if (G == 4) densities64<4>(g, slots, scratch, coef, lane, at_state, duo);
+            else if (G == 8) densities64<8>(g, slots, scratch, coef, lane, at_state, duo);
+            else densities64<16>(g, slots, scratch, coef, lane, at_state, duo);
+            Duo::signal(Duo::kDensity);
+            continue;
+        }
+        const double *ys = duo.sm + (what / Duo::kSingle - 1);
+        density64<32>(g, duo.D[Duo::dXfac], ys, scratch, coef, lane);
         Duo::signal(Duo::kDensity);
         if (g.iso != 0) continue;
         Duo::wait(Duo::kField);
@@ -559,7 +576,7 @@ __device__ __forceinline__ void write_raw(rt_ray_result *out, int id, double P, 
 // them plus 60 trials.
 template <int G>
 __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, double *slots, double *scratch,
-                                         const double *coef, const double *pow2q, int *map, int &n_act,
+                                         const double *pow2q, int *map, int &n_act,
                                          rt_ray_result *__restrict__ out, Duo &duo) {
     const int lane = threadIdx.x, grp = lane / G, q = lane % G;  // the block's first warp
     const bool has = grp < n_act;
@@ -585,6 +602,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
     const int id = SI[kId];
     bool live = has;
     const bool writer = q == 0;
+    if (writer) duo.slot_of[grp] = slot;
     if (G == 32 && writer) duo.D[Duo::dXfac] = rp.xfac;
     __syncwarp();
     for (;;) {
@@ -613,7 +631,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
         // k1 where it is not known (a new state)
         const bool need = live && !(flags & kK1Valid);
         if (__any_sync(kFull, need)) {
-            const double sth = stage64<G>(g, rp, S + kY, C, coef, q, S + kK1, need, duo);
+            const double sth = stage64<G>(rp, S + kY, true, C, q, S + kK1, need, duo);
             if (need) {
                 ++ev;
                 flags |= kK1Valid;
@@ -659,7 +677,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
                                      : fma(s == 3 ? hs : 0.5 * hs, s == 1 ? S[kK1 + c] : C[cK + 6 * (s - 2) + c], y);
             }
             __syncwarp();
-            stage64<G>(g, rp, C + cT, C, coef, q, C + cK + 6 * (s - 1), true, duo);
+            stage64<G>(rp, C + cT, false, C, q, C + cK + 6 * (s - 1), true, duo);
             __syncwarp();
         }
         if (adaptive) {
@@ -790,23 +808,25 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
 
 // Bytes of shared memory of a block that starts with R rays.
 constexpr size_t fp64_smem_bytes(int R) {
-    return sizeof(double) * (size_t)(kPoly + kPow2 + Duo::dSize + R * (kSlot + cGroup)) + (kMaxRays + 1) * sizeof(int);
+    return sizeof(double) * (size_t)(kPoly + kPow2 + Duo::dSize + R * (kSlot + cGroup)) + (2 * kMaxRays + 1) * sizeof(int);
 }
 static_assert(fp64_smem_bytes(kMaxRays) <= 48 * 1024, "fits the default shared-memory limit");
 
 // A warp with R rays (a power of two, at most kMaxRays) at the start and its
-// helper per block.
-__global__ void __launch_bounds__(64) trace_fp64_kernel(const __grid_constant__ GridDev g,
+// helper per block.  Six blocks per SM (168 registers): the FP64 pipe is full
+// with four warps, and more blocks only slow a fan's longest rays (24,840 rays
+// 149 ms, 162 with the eight of 128 registers).
+__global__ void __launch_bounds__(64, 6) trace_fp64_kernel(const __grid_constant__ GridDev g,
                                                         const __grid_constant__ FanDev f, int R,
                                                         rt_ray_result *__restrict__ out) {
     extern __shared__ double sm[];
     double *coef = sm, *pow2q = coef + kPoly, *hand = pow2q + kPow2, *slots = hand + Duo::dSize,
            *scratch = slots + R * kSlot;
     int *map = (int *)(scratch + R * cGroup);
-    Duo duo{hand, map + kMaxRays, sm};
+    Duo duo{hand, map + kMaxRays, map + kMaxRays + 1, sm};
     const int lane = threadIdx.x & 31;
     if (threadIdx.x >= 32) {
-        helper64(g, sm, scratch, coef, lane, duo);
+        helper64(g, slots, scratch, coef, lane, duo);
         return;
     }
     if (lane < kPoly) coef[lane] = (&c_poly[g.interp == 1 ? 1 : 0][0][0])[lane];
@@ -851,12 +871,12 @@ __global__ void __launch_bounds__(64) trace_fp64_kernel(const __grid_constant__ 
     __syncwarp();
     int n_act = __popc(am);
     while (n_act > 0) {
-        if (n_act > 4) run_rays<4>(g, f, slots, scratch, coef, pow2q, map, n_act, out, duo);
-        else if (n_act > 2) run_rays<8>(g, f, slots, scratch, coef, pow2q, map, n_act, out, duo);
-        else if (n_act > 1) run_rays<16>(g, f, slots, scratch, coef, pow2q, map, n_act, out, duo);
-        else run_rays<32>(g, f, slots, scratch, coef, pow2q, map, n_act, out, duo);
+        if (n_act > 4) run_rays<4>(g, f, slots, scratch, pow2q, map, n_act, out, duo);
+        else if (n_act > 2) run_rays<8>(g, f, slots, scratch, pow2q, map, n_act, out, duo);
+        else if (n_act > 1) run_rays<16>(g, f, slots, scratch, pow2q, map, n_act, out, duo);
+        else run_rays<32>(g, f, slots, scratch, pow2q, map, n_act, out, duo);
     }
-    duo.stop(lane);
+    duo.start(0, lane);  // the helper ends
 }
 
 }  // namespace
@@ -865,9 +885,9 @@ __global__ void __launch_bounds__(64) trace_fp64_kernel(const __grid_constant__ 
 // its SM holds fewer than ~3.4 warps and 19 cycles per resident warp above
 // that; kCost is what an evaluation takes in FP64 instructions at 4, 8, 16 and
 // 32 lanes per ray.  The size with the least product is taken.  Measured at 8 /
-// 4 / 2 / 1 rays per warp: 16 rays 54 / 42 / 36 / 25 ms, 522 rays 27 / 22 / 20 /
-// 17 ms, 3,232 rays 45 / 43 / 61 / 95 ms, 4,968 rays 106 / 108 / 113 / 152 ms,
-// 24,840 rays 157 / 214 / 341 ms / -.  More rays per warp (one or two lanes
+// 4 / 2 / 1 rays per warp: 16 rays 47 / 36 / 29 / 25 ms, 522 rays 23 / 18 / 16 /
+// 17 ms, 3,232 rays 40 / 41 / 63 / 96 ms, 4,968 rays 104 / 113 / 129 / 162 ms,
+// 24,840 rays 149 / 208 / 340 ms / -.  More rays per warp (one or two lanes
 // each) were no faster at any size: 24,840 rays 184 ms with 32, 177 with 16,
 // against 174 with 8, all before the second warp.
 int fp64_rays_per_warp(long long n_rays, int sms) {
