@@ -24,8 +24,8 @@
 // (fp64_rays_per_warp).  Measured with one thread per ray / lane groups / and
 // the second warp: 16 rays RK4 without a field 133 / 32 / 24.9 ms, one RKF45
 // ray 42.5 / 16.1 / 11.9 ms (one evaluation 21.2 / 8.0 / 5.9 us), 522 rays - /
-// 19.3 / 16.6 ms, 3,232 rays - / 49.0 / 39.5 ms, the 24,840-ray fan 418 / 172 /
-// 149 ms.
+// 19.3 / 16.6 ms, 3,232 rays - / 49.0 / 39.0 ms, the 24,840-ray fan 418 / 172 /
+// 148 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -63,9 +63,9 @@ enum {
 enum { kId = 0, kMode, kSteps, kAtt, kEv, kFlags, kSide, kIt };
 enum { kK1Valid = 1, kHavePrev = 2, kLands = 4, kExits = 8 };
 // Scratch (one per group): derivatives k2..k6, stage state / new state, error
-// estimate, in-cell coordinates and cells of the three axes, the 24 weights,
+// estimate, in-cell coordinates t and 1 - t and cells of the three axes, the 24 weights,
 // the altitude, longitude and latitude sums.
-enum { cK = 0, cT = 30, cE = 36, cFrac = 42, cCell = 45 /* 3 ints */, cW = 47, cV = 71, cS = 103, cO = 115, cGroup = 119 };
+enum { cK = 0, cT = 30, cE = 36, cFrac = 42, cCell = 48 /* 3 ints */, cW = 50, cV = 74, cS = 106, cO = 118, cGroup = 123 };
 static_assert(kSlot % 2 == 1 && cGroup % 2 == 1, "odd strides spread the groups over the banks");
 constexpr int kMaxRays = 8;  // rays a warp starts with at most (G = 4)
 constexpr int kPoly = 4 * 5, kPow2 = 20;  // tables at the start of the shared memory
@@ -387,6 +387,7 @@ __device__ __forceinline__ void density64(const GridDev &g, double xfac, const d
         double t;
         const bool ok = cell64(grid_coord64(g, q, ys[0], ys[1], ys[2]), q == 0 ? g.n_lat : q == 1 ? g.n_lon : g.n_alt, i, t);
         C[cFrac + q] = t;
+        C[cFrac + 3 + q] = 1.0 - t;
         cell[q] = ok ? i : -1;
     }
     __syncwarp();
@@ -402,8 +403,7 @@ __device__ __forceinline__ void density64(const GridDev &g, double xfac, const d
         const bool right = node >= 2;
         const bool outer = node == 0 || node == 3;  // nodes j-1, j+2
         const double *cf = coef + (der * 2 + (outer ? 0 : 1)) * 5;
-        double t = C[cFrac + (p >> 3)];
-        t = right ? 1.0 - t : t;
+        const double t = C[cFrac + (right ? 3 : 0) + (p >> 3)];
         double w = fma(t, cf[0], cf[1]);
         w = fma(t, w, cf[2]);
         w = fma(t, w, cf[3]);
