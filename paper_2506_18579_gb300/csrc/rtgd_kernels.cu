@@ -736,18 +736,21 @@ __global__ void finish_fans_records_kernel(double R_E, const FanDev *__restrict_
                   r.n_steps, r.n_attempts, r.n_evals, R_E, out + i);
 }
 
-// Once k1 is known: end an adaptive step just past the next cell face, and
-// clip it at the group-path limit.
-__device__ __forceinline__ void lane_limit_step(Lane &L, const GridDev &g, const FanDev &f) {
-    if (L.landing) return;
+// Once k1 is known: the accumulators start from it, an adaptive step ends just
+// past the next cell face, and the group-path limit clips it.  The
+// accumulation's 42 products stand in the face distance's block, beside its
+// divisions.
+__device__ __forceinline__ void lane_limit_step(Lane &L, const GridDev &g, const FanDev &f, const Tableau &T) {
     if (f.integrator == RT_RKF45) {
         const float hf = face_distance_f(g, L.b, L.k1);
-        if (hf > 1e-3f * L.hs && hf < L.hs) {
-            L.hs = hf * (1.0f + 1e-4f);
-            L.at_face = true;
-        }
+        accumulate_first(L, T, L.k1);
+        const bool cut = !L.landing && hf > 1e-3f * L.hs && hf < L.hs;
+        L.hs = cut ? hf * (1.0f + 1e-4f) : L.hs;
+        L.at_face = L.at_face || cut;
+    } else {
+        accumulate_first(L, T, L.k1);
     }
-    if (f.has_max_path) {
+    if (f.has_max_path && !L.landing) {
         const double P = L.P + ((double)L.inc_hi[3] + (double)L.inc_lo[3]);
         if (P + (double)L.hs > f.max_path) L.hs = (float)(f.max_path - P);
     }
@@ -808,8 +811,7 @@ __device__ __forceinline__ void lane_stage0_done(Lane &L, const GridDev &g, cons
         }
         L.have_prev = false;
     }
-    lane_limit_step(L, g, f);
-    accumulate_first(L, T, L.k1);
+    lane_limit_step(L, g, f, T);
 }
 
 // The stages of one step attempt.  Every lane of a warp runs its attempt in
