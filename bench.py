@@ -38,7 +38,7 @@ METRIC = "rays/s and ray-steps/s at ≤0.05 km P'/D error; p50/p99 fan latency"
 # counts 2): GD weights 3 x 37 FMA, contraction 192 FMA, grid-coordinate and
 # chain factors ~20 flop, dipole + Jacobian ~70, Appleton-Hartree + partials
 # ~60, Hamiltonian partials + ray equations ~70, stage offsets and RK
-# accumulation ~90 (mixed path; the FP64 path accumulates inside rk*_step64).
+# accumulation ~90 (mixed path; the FP64 path: rkf45_stage).
 FLOP_PER_EVAL = {"mixed": 1000.0, "fp64": 910.0}
 # Grid samples one stage evaluation reads: 64 samples (16 rows of 4) plus the
 # reference node, FP32 in the mixed path and FP64 in the all-FP64 path.
@@ -48,18 +48,19 @@ GATHER_BYTES = {"mixed": 65 * 4, "fp64": 64 * 8}
 # L2 flush between timed steps), keyed by workload and launch configuration
 # (kernel, stencil, lanes per ray) and valid only for the kernel sources it
 # was captured from: a changed kernel reports traffic null.
-KERNEL_SOURCES = ("paper_2506_18579_gb300/csrc/rtgd_kernels.cu", "paper_2506_18579_gb300/csrc/rtgd_device.cuh")
+KERNEL_SOURCES = tuple("paper_2506_18579_gb300/csrc/" + f for f in (
+    "rtgd_kernels.cu", "rtgd_device.cuh", "rtgd_fan.cuh", "rtgd_fp64.cuh"))
 TRAFFIC = {
     # key = (workload, kernel, stencil, lanes per ray); the anisotropic fan in
     # the autotuner's configurations (plain, 4 lanes, 96-thread blocks)
-    ("c2", 1, 3, 4): {"bytes_per_launch": 26831616 + 22528, "source_sha256": "2602d2aac951aea9"},
-    ("c2", 1, 2, 4): {"bytes_per_launch": 5379072 + 256, "source_sha256": "2602d2aac951aea9"},
+    ("c2", 1, 3, 4): {"bytes_per_launch": 27159040 + 85504, "source_sha256": "4b77e02ae9a043ad"},
+    ("c2", 1, 2, 4): {"bytes_per_launch": 5581824 + 27904, "source_sha256": "4b77e02ae9a043ad"},
     # the ionogram batch, one lane per ray (the only lane count the autotuner
     # tries on a fan this large): plain kernel with 32-thread blocks (table
     # and quad stencils), persistent kernel with 128-thread blocks
-    ("c4", 1, 3, 1): {"bytes_per_launch": 21227520 + 1478144, "source_sha256": "2602d2aac951aea9"},
-    ("c4", 1, 2, 1): {"bytes_per_launch": 4333312 + 483584, "source_sha256": "2602d2aac951aea9"},
-    ("c4", 2, 3, 1): {"bytes_per_launch": 20590080 + 385792, "source_sha256": "2602d2aac951aea9"},
+    ("c4", 1, 3, 1): {"bytes_per_launch": 20942848 + 2286080, "source_sha256": "4b77e02ae9a043ad"},
+    ("c4", 1, 2, 1): {"bytes_per_launch": 4317952 + 1300224, "source_sha256": "4b77e02ae9a043ad"},
+    ("c4", 2, 3, 1): {"bytes_per_launch": 20998144 + 1057792, "source_sha256": "4b77e02ae9a043ad"},
 }
 SMS = 152
 FP32_LANES_PER_SM = 128
