@@ -53,14 +53,14 @@ KERNEL_SOURCES = tuple("paper_2506_18579_gb300/csrc/" + f for f in (
 TRAFFIC = {
     # key = (workload, kernel, stencil, lanes per ray); the anisotropic fan in
     # the autotuner's configurations (plain, 4 lanes, 96-thread blocks)
-    ("c2", 1, 3, 4): {"bytes_per_launch": 27159040 + 85504, "source_sha256": "4b77e02ae9a043ad"},
-    ("c2", 1, 2, 4): {"bytes_per_launch": 5581824 + 27904, "source_sha256": "4b77e02ae9a043ad"},
+    ("c2", 1, 3, 4): {"bytes_per_launch": 27159040 + 85504, "source_sha256": "fa834026b2b0187e"},
+    ("c2", 1, 2, 4): {"bytes_per_launch": 5581824 + 27904, "source_sha256": "fa834026b2b0187e"},
     # the ionogram batch, one lane per ray (the only lane count the autotuner
     # tries on a fan this large): plain kernel with 32-thread blocks (table
     # and quad stencils), persistent kernel with 128-thread blocks
-    ("c4", 1, 3, 1): {"bytes_per_launch": 20942848 + 2286080, "source_sha256": "4b77e02ae9a043ad"},
-    ("c4", 1, 2, 1): {"bytes_per_launch": 4317952 + 1300224, "source_sha256": "4b77e02ae9a043ad"},
-    ("c4", 2, 3, 1): {"bytes_per_launch": 20998144 + 1057792, "source_sha256": "4b77e02ae9a043ad"},
+    ("c4", 1, 3, 1): {"bytes_per_launch": 20942848 + 2286080, "source_sha256": "fa834026b2b0187e"},
+    ("c4", 1, 2, 1): {"bytes_per_launch": 4317952 + 1300224, "source_sha256": "fa834026b2b0187e"},
+    ("c4", 2, 3, 1): {"bytes_per_launch": 20998144 + 1057792, "source_sha256": "fa834026b2b0187e"},
 }
 SMS = 152
 FP32_LANES_PER_SM = 128

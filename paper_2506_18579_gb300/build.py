@@ -1,6 +1,6 @@
 """Builds librtgd.so in-tree with nvcc for sm_103a (GB300).
 
-Two translation units compiled in parallel, then linked into a shared
+Its translation units are compiled in parallel, then linked into a shared
 library next to this file.  Rebuilds only when a source or header is newer
 than the library.
 """

@@ -210,7 +210,7 @@ rt_err make_plan(const rt_grid *grid, const rt_fan_desc *fan, size_t n_rays, con
     }
     if (c.kernel == RT_KERNEL_AUTO) c.kernel = RT_KERNEL_PLAIN;  // measured faster on GB300 for small and large fans
     if (fan->precision == RT_FP64 && c.kernel != RT_KERNEL_PLAIN)
-        return fail(RT_EINVAL, "the FP64 path runs the plain one-thread-per-ray kernel only");
+        return fail(RT_EINVAL, "the FP64 path has the plain kernel only");
     if (c.stencil == RT_STENCIL_AUTO) c.stencil = RT_STENCIL_QUAD;
     if (c.stencil == RT_STENCIL_TABLE && !grid->table)
         return fail(RT_EINVAL, "stencil TABLE needs a grid created with RT_GRID_TABLE");
@@ -222,7 +222,7 @@ rt_err make_plan(const rt_grid *grid, const rt_fan_desc *fan, size_t n_rays, con
     if (c.stencil == RT_STENCIL_GATHER && c.kernel == RT_KERNEL_PLAIN) c.stencil = RT_STENCIL_QUAD;
     if (c.order == RT_ORDER_CANONICAL && cfg == nullptr) c.order = RT_ORDER_ELEVATION_FASTEST;
     if (fan->precision == RT_FP64 && c.lanes_per_ray > 1)
-        return fail(RT_EINVAL, "the FP64 path runs one lane per ray");
+        return fail(RT_EINVAL, "lanes_per_ray does not apply to the FP64 path");
     lp->kernel = c.kernel;
     lp->stencil = c.stencil;
     lp->threads = c.block_threads ? c.block_threads : 128;

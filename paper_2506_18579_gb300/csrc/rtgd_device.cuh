@@ -1,7 +1,7 @@
 // rtgd_device.cuh -- device-side building blocks of the RTM-GD tracer.
 //
-// Everything the stage evaluation needs, written once and instantiated for
-// double (the all-FP64 path) and float (the mixed path):
+// What the stage evaluation needs (weights and contraction for float and
+// double; the physics for float, the FP64 path's is tail64 in rtgd_fp64.cuh):
 //   - p = 3 Galerkin-Difference weights and their derivatives (Appendix A),
 //   - the 4x4x4 tensor contraction of Eq. 13 giving Ne and its gradient,
 //   - the centred dipole field and its Jacobian in local spherical components,
@@ -197,32 +197,16 @@ __device__ __forceinline__ void acc_row(R v, R dv, R wb, R db, R &s, R &sb, R &s
         out[3] = nc_;                                                             \
     } while (0)
 
-// 1/x: correctly rounded in double; in float the fast reciprocal (MUFU.RCP,
-// within 2 ulp), which is ample for the mixed path's tolerance.
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+// 1/x: the fast reciprocal (MUFU.RCP, within 2 ulp), which is ample for the
+// mixed path's tolerance.
 __device__ __forceinline__ float recip(float x) { return __fdividef(1.0f, x); }
 
-// sqrt: correctly rounded in double; in float x * rsqrt(x) (MUFU.RSQ, a few
-// ulp, no special-case branch), 0 for x <= 0.
-__device__ __forceinline__ double fsqrt(double x) { return sqrt(x); }
+// sqrt: x * rsqrt(x) (MUFU.RSQ, a few ulp, no special-case branch), 0 for x <= 0.
 __device__ __forceinline__ float fsqrt(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
 
-// a / b: correctly rounded in double; in float the fast division (MUFU.RCP
-// based, 2 ulp, no special-case branch) for the step-control arithmetic.
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
+// a / b: the fast division (MUFU.RCP based, 2 ulp, no special-case branch) for
+// the step-control arithmetic.
 __device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-
-// Cell index and local coordinate along one axis; false outside [0, n-1].
-template <typename R>
-__device__ __forceinline__ bool cell_coord(R x, int n, int &i, R &t) {
-    if (!(x >= R(0) && x <= R(n - 1))) return false;
-    R f = floor(x);
-    int fi = (int)f;
-    if (fi > n - 2) fi = n - 2;
-    i = fi;
-    t = x - R(fi);
-    return true;
-}
 
 // --------------------------------------------------------------------------
 // Physics at one stage: everything after the interpolation.

@@ -4,7 +4,7 @@
 //                       (4 consecutive altitude samples per float4) and the
 //                       optional per-cell 64-sample table (Sec. II-C: the
 //                       interpolation data are prepared once per grid cell).
-//   trace_fp64        : all-FP64 tracer, one thread per ray.
+//                       (The all-FP64 tracer is in rtgd_fp64.cu.)
 //   trace_mixed_*     : mixed-precision tracer.  A group of 1, 2 or 4 lanes
 //                       carries one ray; every loop iteration runs one whole
 //                       RK attempt for all lanes of a warp (the stage index
