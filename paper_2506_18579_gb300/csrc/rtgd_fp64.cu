@@ -24,8 +24,8 @@
 // (fp64_rays_per_warp).  Measured with one thread per ray / lane groups / and
 // the second warp: 16 rays RK4 without a field 133 / 32 / 24.9 ms, one RKF45
 // ray 42.5 / 16.1 / 11.9 ms (one evaluation 21.2 / 8.0 / 5.9 us), 522 rays - /
-// 19.3 / 16.6 ms, 3,232 rays - / 49.0 / 39.0 ms, the 24,840-ray fan 418 / 172 /
-// 148 ms.
+// 19.3 / 16.6 ms, 3,232 rays - / 49.0 / 38.4 ms, the 24,840-ray fan 418 / 172 /
+// 147 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -397,6 +397,18 @@ __device__ __forceinline__ void density64(const GridDev &g, double xfac, const d
         if (q < 4) C[cO + q] = 0.0;
         return;
     }
+    // this lane's sample rows, loaded ahead of the weights that they wait for
+    constexpr int kRows = G == 32 ? 1 : 16 / G;
+    const long long sj = g.p_alt, si = (long long)g.p_lon * g.p_alt;
+    const double *base = g.pad64 + (long long)(inside ? ca : 0) * si + (long long)(inside ? cb : 0) * sj + (inside ? cc : 0);
+    double u[kRows][4];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const int row = G == 32 ? (q & 15) : q + r * G;
+        const double *p = base + (row >> 2) * si + (row & 3) * sj;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) u[r][c] = __ldg(p + c);
+    }
     // the 24 weights: weight p = 8 axis + 4 derivative + node, one polynomial each
     for (int p = q; p < 24; p += G) {
         const int node = p & 3, der = (p >> 2) & 1;
@@ -414,21 +426,17 @@ __device__ __forceinline__ void density64(const GridDev &g, double xfac, const d
         C[cW + p] = (der && right) ? -w : w;
     }
     __syncwarp();
-    const long long sj = g.p_alt, si = (long long)g.p_lon * g.p_alt;
-    const double *base = g.pad64 + (long long)(inside ? ca : 0) * si + (long long)(inside ? cb : 0) * sj + (inside ? cc : 0);
     // altitude rows (Eq. 13): row 4 a + b; with 32 lanes the upper half forms the derivative sums
     if (G == 32) {
-        const int row = q & 15;
-        const double *p = base + (row >> 2) * si + (row & 3) * sj;
         const double *w = C + cW + 16 + ((q >> 4) << 2);
-        C[cV + q] = fma(__ldg(p + 3), w[3], fma(__ldg(p + 2), w[2], fma(__ldg(p), w[0], __dmul_rn(__ldg(p + 1), w[1]))));
+        C[cV + q] = fma(u[0][3], w[3], fma(u[0][2], w[2], fma(u[0][0], w[0], __dmul_rn(u[0][1], w[1]))));
     } else {
-        for (int row = q; row < 16; row += G) {
-            const double *p = base + (row >> 2) * si + (row & 3) * sj;
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
             double v, dv;
-            row4<double>(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3), C + cW + 16, C + cW + 20, v, dv);
-            C[cV + row] = v;
-            C[cV + 16 + row] = dv;
+            row4<double>(u[r][0], u[r][1], u[r][2], u[r][3], C + cW + 16, C + cW + 20, v, dv);
+            C[cV + q + r * G] = v;
+            C[cV + 16 + q + r * G] = dv;
         }
     }
     __syncwarp();
