@@ -21,11 +21,14 @@
 // perform them change), so its record depends neither on G nor on its warp
 // mates.  Ray states live in shared memory (slots), so that regrouping moves
 // no data.  The host starts a warp with as many rays as fill the GPU
-// (fp64_rays_per_warp).  Measured with one thread per ray / lane groups / and
+// (fp64_rays_per_warp); a fan that fills it many times over starts with 32 rays
+// a warp, one per lane (~770 instructions for 32 evaluations, the groups of
+// four lanes ~260 for eight), and goes over to groups once 16 are left, eight of
+// those at a time.  Measured with one thread per ray / lane groups / and
 // the second warp: 16 rays RK4 without a field 133 / 32 / 24.9 ms, one RKF45
 // ray 42.5 / 16.1 / 11.9 ms (one evaluation 21.2 / 8.0 / 5.9 us), 522 rays - /
 // 19.3 / 16.6 ms, 3,232 rays - / 49.0 / 38.4 ms, the 24,840-ray fan 418 / 172 /
-// 147 ms.
+// 147 ms; 495,122 rays 2,026 ms, 2,551 from eight rays a warp and 1,535 from 32.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -37,21 +40,6 @@ namespace rtgd {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-
-// Polynomials of the one-dimensional weights (Appendix A; Eq. 7 for
-// Catmull-Rom) as Horner coefficients, highest power first: kinds 0 and 1
-// are the weights of nodes j-1 and j, kinds 2 and 3 their derivatives.
-//   kind 0: t p4(t), kind 1: 1 + t^2 p3(t), kind 2: p4(t), kind 3: t p3(t)
-// with p4 of all five coefficients and p3 of the first four.
-__constant__ double c_poly[2][4][5] = {
-    {{1.0 / 6.0, -5.0 / 12.0, -1.0 / 6.0, 11.0 / 12.0, -0.5},
-     {-0.5, 1.25, 0.5, -2.25, 0.0},
-     {5.0 / 6.0, -5.0 / 3.0, -0.5, 11.0 / 6.0, -0.5},
-     {-2.5, 5.0, 1.5, -4.5, 0.0}},
-    {{0.0, 0.0, -0.5, 1.0, -0.5},
-     {0.0, 0.0, 1.5, -2.5, 0.0},
-     {0.0, 0.0, -1.5, 2.0, -0.5},
-     {0.0, 0.0, 4.5, -5.0, 0.0}}};
 
 // Shared memory of a block, in doubles.  Slot (one per ray): state, k1,
 // sin(theta) at the state, then the scalars below.
@@ -66,8 +54,17 @@ enum { kK1Valid = 1, kHavePrev = 2, kLands = 4, kExits = 8 };
 // estimate, in-cell coordinates t and 1 - t and cells of the three axes, the 24 weights,
 // the altitude, longitude and latitude sums.
 enum { cK = 0, cT = 30, cE = 36, cFrac = 42, cCell = 48 /* 3 ints */, cW = 50, cV = 74, cS = 106, cO = 118, cGroup = 123 };
-static_assert(kSlot % 2 == 1 && cGroup % 2 == 1, "odd strides spread the groups over the banks");
-constexpr int kMaxRays = 8;  // rays a warp starts with at most (G = 4)
+// One lane per ray: the derivatives, the stage state and the error estimate only.
+enum { cLane = 43 };
+static_assert(kSlot % 2 == 1 && cGroup % 2 == 1 && cLane % 2 == 1 && cLane >= cFrac, "odd strides spread the groups over the banks");
+constexpr int kGroups = 8;    // groups of a warp at most (G = 4)
+constexpr int kBlocksPerSm = 6;
+constexpr int kWideRays = 32;  // rays that a warp of the wide kernel starts with
+// One lane per ray until this few are left.  Eight of 16 at a time cost the pipe
+// what 16 lanes of their own do, and take a cluster of long rays to its end
+// sooner.  Measured at 8 / 16 / 20 / 24: 24,840 rays 148 / 152 / 160 / 162 ms,
+// 100,434 rays 564 / 483 / 490 / 493 ms, 248,442 rays 775 / 788 / 797 / 824 ms.
+constexpr int kWideLeft = 16;
 constexpr int kPoly = 4 * 5, kPow2 = 20;  // tables at the start of the shared memory
 
 __device__ __noinline__ double div_rare(double x, double c) { return x / c; }
@@ -429,14 +426,12 @@ __device__ __forceinline__ void density64(const GridDev &g, double xfac, const d
     // altitude rows (Eq. 13): row 4 a + b; with 32 lanes the upper half forms the derivative sums
     if (G == 32) {
         const double *w = C + cW + 16 + ((q >> 4) << 2);
-        C[cV + q] = fma(u[0][3], w[3], fma(u[0][2], w[2], fma(u[0][0], w[0], __dmul_rn(u[0][1], w[1]))));
+        C[cV + q] = row64(u[0][0], u[0][1], u[0][2], u[0][3], w);
     } else {
 #pragma unroll
         for (int r = 0; r < kRows; ++r) {
-            double v, dv;
-            row4<double>(u[r][0], u[r][1], u[r][2], u[r][3], C + cW + 16, C + cW + 20, v, dv);
-            C[cV + q + r * G] = v;
-            C[cV + 16 + q + r * G] = dv;
+            C[cV + q + r * G] = row64(u[r][0], u[r][1], u[r][2], u[r][3], C + cW + 16);
+            C[cV + 16 + q + r * G] = row64(u[r][0], u[r][1], u[r][2], u[r][3], C + cW + 20);
         }
     }
     __syncwarp();
@@ -447,7 +442,7 @@ __device__ __forceinline__ void density64(const GridDev &g, double xfac, const d
         const double *w = C + cW + 8 + (j == 1 ? 4 : 0);
         double sum = 0.0;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) sum += v[b] * w[b];
+        for (int b = 0; b < 4; ++b) sum = fma(v[b], w[b], sum);
         C[cS + id] = sum;
     }
     __syncwarp();
@@ -457,7 +452,7 @@ __device__ __forceinline__ void density64(const GridDev &g, double xfac, const d
         const double *w = C + cW + (o == 1 ? 4 : 0);
         double sum = 0.0;
 #pragma unroll
-        for (int a = 0; a < 4; ++a) sum += v[3 * a] * w[a];
+        for (int a = 0; a < 4; ++a) sum = fma(v[3 * a], w[a], sum);
         const double c1 = o == 0 ? 1.0 : o == 1 ? g.inv_dlat : o == 2 ? g.inv_dlon : g.inv_dalt;
         const double c2 = o == 1 || o == 2 ? kRad2Deg : 1.0;
         C[cO + o] = inside ? (o == 1 ? -xfac : xfac) * sum * c1 * c2 : 0.0;
@@ -486,9 +481,21 @@ __device__ __forceinline__ void angles64(StageIn<double> &s, const double *ys, i
 // this one forms the sines, the field and Appleton-Hartree's arguments, and
 // with 32 lanes the field's gradients while this one goes through
 // Appleton-Hartree.
+// G = 1: the lane evaluates alone, the second warp does nothing.
 template <int G>
-__device__ __forceinline__ double stage64(const RayPhys<double> &rp, const double *ys, bool at_state, const double *C,
-                                          int q, double *out, bool write, Duo &duo) {
+__device__ __forceinline__ double stage64(const GridDev &g, const RayPhys<double> &rp, const double *ys, bool at_state,
+                                          const double *C, int q, double *out, bool write, Duo &duo) {
+    if constexpr (G == 1) {
+        double y[6], dy[6], sth;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) y[i] = ys[i];
+        rhs64(g, rp, y, dy, nullptr, &sth);
+        if (write) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) out[i] = dy[i];
+        }
+        return sth;
+    }
     StageIn<double> s;
     const int j = (q & 3) == 3 ? 2 : (q & 3);  // the component this lane carries
     double d, dk;
@@ -576,7 +583,7 @@ __device__ __forceinline__ void write_raw(rt_ray_result *out, int id, double P, 
 }
 
 // Runs the warp's rays, G lanes each, until at most half of the groups are
-// still in use; then packs the remaining rays' slots to the front of map.
+// still in use (G = 1: until kWideLeft rays are left); then packs the remaining rays' slots to the front of map.
 // One iteration is one step attempt (or one trial of the landing / exit
 // solve) of every ray.  Groups without a ray follow group 0's ray and write
 // nothing, so that the warp's barriers stay uniform.  The loop ends: every
@@ -591,7 +598,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
     const int slot = map[has ? grp : 0];
     double *S = slots + slot * kSlot;
     int *SI = (int *)(S + kInts);
-    double *C = scratch + grp * cGroup;
+    double *C = scratch + grp * (G == 1 ? cLane : cGroup);
     const bool adaptive = f.integrator == RT_RKF45;
     const int ns = adaptive ? 6 : 4;
     const double RE = g.R_E;
@@ -610,13 +617,13 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
     const int id = SI[kId];
     bool live = has;
     const bool writer = q == 0;
-    if (writer) duo.slot_of[grp] = slot;
+    if (G > 1 && writer) duo.slot_of[grp] = slot;
     if (G == 32 && writer) duo.D[Duo::dXfac] = rp.xfac;
     __syncwarp();
     for (;;) {
         const unsigned am = __ballot_sync(kFull, live && writer);
         const int n = __popc(am);
-        if (n == 0 || (G < 32 && 2 * n * G <= 32)) {
+        if (n == 0 || (G == 1 ? n <= kWideLeft : G < 32 && 2 * n * G <= 32)) {
             if (live && writer) {
                 S[kP] = P; S[kH] = h; S[kHs] = hs; S[kApo] = apo; S[kRPrev] = r_prev; S[kDrPrev] = dr_prev;
                 S[kHPrev] = h_prev; S[kLa] = la; S[kLfa] = lfa; S[kLb] = lb; S[kLfb] = lfb;
@@ -639,7 +646,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
         // k1 where it is not known (a new state)
         const bool need = live && !(flags & kK1Valid);
         if (__any_sync(kFull, need)) {
-            const double sth = stage64<G>(rp, S + kY, true, C, q, S + kK1, need, duo);
+            const double sth = stage64<G>(g, rp, S + kY, true, C, q, S + kK1, need, duo);
             if (need) {
                 ++ev;
                 flags |= kK1Valid;
@@ -653,16 +660,26 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
             // distance to the next cell face, predicted linearly from k1; lateral
             // faces count only inside the altitude span
             const double y0 = S[kY], y1 = S[kY + 1], y2 = S[kY + 2];
-            const int ax = (q & 3) == 3 ? 2 : (q & 3);  // an axis per lane
-            const double x = grid_coord64(g, ax, y0, y1, y2);
-            const double v = (ax == 0 ? -S[kK1 + 1] : ax == 1 ? S[kK1 + 2] : S[kK1]) * (ax == 2 ? 1.0 : kRad2Deg) *
-                             (ax == 0 ? g.inv_dlat : ax == 1 ? g.inv_dlon : g.inv_dalt);
-            const double xc = __shfl_sync(kFull, x, 2, 4);
-            const bool in_alt = xc >= 0.0 && xc <= (double)(g.n_alt - 1);
-            double best = face_axis64(x, v, ax == 0 ? g.n_lat : ax == 1 ? g.n_lon : g.n_alt);
-            if (ax < 2 && !in_alt) best = HUGE_VAL;
-            best = fmin(best, __shfl_xor_sync(kFull, best, 1));
-            best = fmin(best, __shfl_xor_sync(kFull, best, 2));
+            auto face = [&](int ax, double &x) {
+                x = grid_coord64(g, ax, y0, y1, y2);
+                const double v = (ax == 0 ? -S[kK1 + 1] : ax == 1 ? S[kK1 + 2] : S[kK1]) * (ax == 2 ? 1.0 : kRad2Deg) *
+                                 (ax == 0 ? g.inv_dlat : ax == 1 ? g.inv_dlon : g.inv_dalt);
+                return face_axis64(x, v, ax == 0 ? g.n_lat : ax == 1 ? g.n_lon : g.n_alt);
+            };
+            double x, best;
+            if constexpr (G == 1) {
+                const double d0 = face(0, x), d1 = face(1, x), d2 = face(2, x);
+                const bool in_alt = x >= 0.0 && x <= (double)(g.n_alt - 1);
+                best = in_alt ? fmin(fmin(d0, d1), d2) : d2;
+            } else {
+                const int ax = (q & 3) == 3 ? 2 : (q & 3);  // an axis per lane
+                best = face(ax, x);
+                const double xc = __shfl_sync(kFull, x, 2, 4);
+                const bool in_alt = xc >= 0.0 && xc <= (double)(g.n_alt - 1);
+                if (ax < 2 && !in_alt) best = HUGE_VAL;
+                best = fmin(best, __shfl_xor_sync(kFull, best, 1));
+                best = fmin(best, __shfl_xor_sync(kFull, best, 2));
+            }
             if (!solving && best > 1e-3 * hs && best < hs) {
                 hs = best * (1.0 + 1e-4);
                 at_face = true;
@@ -685,7 +702,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
                                      : fma(s == 3 ? hs : 0.5 * hs, s == 1 ? S[kK1 + c] : C[cK + 6 * (s - 2) + c], y);
             }
             __syncwarp();
-            stage64<G>(rp, C + cT, false, C, q, C + cK + 6 * (s - 1), true, duo);
+            stage64<G>(g, rp, C + cT, false, C, q, C + cK + 6 * (s - 1), true, duo);
             __syncwarp();
         }
         if (adaptive) {
@@ -720,8 +737,13 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
                 kerr = max3_rare(e3, e4, e5);
             }
             const double dp = f.atol + f.rtol * r, dk = f.rtol * fmax(kmag, 1e-3);
-            const double v = ((q & 1) ? kerr : pos) / ((q & 1) ? dk : dp);
-            const double err = fmax(v, __shfl_xor_sync(kFull, v, 1));
+            double err;
+            if constexpr (G == 1) {
+                err = fmax(pos / dp, kerr / dk);
+            } else {
+                const double v = ((q & 1) ? kerr : pos) / ((q & 1) ? dk : dp);
+                err = fmax(v, __shfl_xor_sync(kFull, v, 1));
+            }
             fac = step_factor64(err, pow2q);
             accept = err <= 1.0;
         }
@@ -729,7 +751,11 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
         int cell_i;
         double cell_t;
         const bool in_ax = cell64(grid_coord64(g, q & 1, yn[0], yn[1], yn[2]), (q & 1) ? g.n_lon : g.n_lat, cell_i, cell_t);
-        const bool lateral = __shfl_xor_sync(kFull, (int)in_ax, 1) && in_ax;
+        bool lateral;
+        if constexpr (G == 1)
+            lateral = cell64(grid_coord64(g, 1, yn[0], yn[1], yn[2]), g.n_lon, cell_i, cell_t) && in_ax;
+        else
+            lateral = __shfl_xor_sync(kFull, (int)in_ax, 1) && in_ax;
         const double y0 = S[kY];
         if (solving) {
             // ground return or exit through the grid top: r(step(h*)) = R_E (or
@@ -815,23 +841,29 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
 }
 
 // Bytes of shared memory of a block that starts with R rays.
-constexpr size_t fp64_smem_bytes(int R) {
-    return sizeof(double) * (size_t)(kPoly + kPow2 + Duo::dSize + R * (kSlot + cGroup)) + (2 * kMaxRays + 1) * sizeof(int);
+__host__ __device__ constexpr int fp64_scratch(int R) {
+    return R <= kGroups ? R * cGroup : R * cLane > kGroups * cGroup ? R * cLane : kGroups * cGroup;
 }
-static_assert(fp64_smem_bytes(kMaxRays) <= 48 * 1024, "fits the default shared-memory limit");
+constexpr size_t fp64_smem_bytes(int R) {
+    return sizeof(double) * (size_t)(kPoly + kPow2 + Duo::dSize + R * kSlot + fp64_scratch(R)) +
+           (R + 1 + kGroups) * sizeof(int);
+}
+static_assert(fp64_smem_bytes(kGroups) <= 48 * 1024 && fp64_smem_bytes(kWideRays) <= 48 * 1024,
+              "fits the default shared-memory limit");
 
-// A warp with R rays (a power of two, at most kMaxRays) at the start and its
-// helper per block.  Six blocks per SM (168 registers): the FP64 pipe is full
-// with four warps, and more blocks only slow a fan's longest rays (24,840 rays
-// 149 ms, 162 with the eight of 128 registers).
-__global__ void __launch_bounds__(64, 6) trace_fp64_kernel(const __grid_constant__ GridDev g,
+// A warp with R rays (a power of two, at most kGroups; WIDE: kWideRays) at the
+// start and its helper per block.  kBlocksPerSm = 6 blocks per SM (168 registers): the FP64
+// pipe is full with four warps, and more blocks only slow a fan's longest rays
+// (24,840 rays 149 ms, 162 with the eight of 128 registers).
+template <bool WIDE>
+__global__ void __launch_bounds__(64, kBlocksPerSm) trace_fp64_kernel(const __grid_constant__ GridDev g,
                                                         const __grid_constant__ FanDev f, int R,
                                                         rt_ray_result *__restrict__ out) {
     extern __shared__ double sm[];
     double *coef = sm, *pow2q = coef + kPoly, *hand = pow2q + kPow2, *slots = hand + Duo::dSize,
            *scratch = slots + R * kSlot;
-    int *map = (int *)(scratch + R * cGroup);
-    Duo duo{hand, map + kMaxRays, map + kMaxRays + 1, sm};
+    int *map = (int *)(scratch + fp64_scratch(R));
+    Duo duo{hand, map + R, map + R + 1, sm};
     const int lane = threadIdx.x & 31;
     if (threadIdx.x >= 32) {
         helper64(g, slots, scratch, coef, lane, duo);
@@ -879,10 +911,17 @@ __global__ void __launch_bounds__(64, 6) trace_fp64_kernel(const __grid_constant
     __syncwarp();
     int n_act = __popc(am);
     while (n_act > 0) {
-        if (n_act > 4) run_rays<4>(g, f, slots, scratch, pow2q, map, n_act, out, duo);
-        else if (n_act > 2) run_rays<8>(g, f, slots, scratch, pow2q, map, n_act, out, duo);
-        else if (n_act > 1) run_rays<16>(g, f, slots, scratch, pow2q, map, n_act, out, duo);
-        else run_rays<32>(g, f, slots, scratch, pow2q, map, n_act, out, duo);
+        if (WIDE && n_act > kWideLeft) {
+            run_rays<1>(g, f, slots, scratch, pow2q, map, n_act, out, duo);
+            continue;
+        }
+        const int wait = WIDE && n_act > kGroups ? n_act - kGroups : 0;  // rays at the front of map whose turn comes later
+        int n = n_act - wait;
+        if (n > 4) run_rays<4>(g, f, slots, scratch, pow2q, map + wait, n, out, duo);
+        else if (n > 2) run_rays<8>(g, f, slots, scratch, pow2q, map + wait, n, out, duo);
+        else if (n > 1) run_rays<16>(g, f, slots, scratch, pow2q, map + wait, n, out, duo);
+        else run_rays<32>(g, f, slots, scratch, pow2q, map + wait, n, out, duo);
+        n_act = wait + n;
     }
     duo.start(0, lane);  // the helper ends
 }
@@ -898,12 +937,23 @@ __global__ void __launch_bounds__(64, 6) trace_fp64_kernel(const __grid_constant
 // 24,840 rays 149 / 208 / 340 ms / -.  More rays per warp (one or two lanes
 // each) were no faster at any size: 24,840 rays 184 ms with 32, 177 with 16,
 // against 174 with 8, all before the second warp.
+//
+// From two full waves of 32-ray warps (58,368 rays on 152 SMs) a fan is bound by
+// the pipe's throughput rather than by its longest rays, and one lane per ray
+// costs the least of it.  One thread per ray to the end / 8 rays / 32 rays per
+// warp: 49,464 short uneven rays (20-28 MHz) 206 / 205 / 140 ms, 61,830 of them
+// 211 / 252 / 174 ms, 98,928 of them 321 / 392 / 254 ms, 98,928 rays of 8-16 MHz
+// 543 / 444 / 325 ms; an elevation scan at 0.1 degrees, whose long rays are
+// neighbours: 51,098 rays 631 / 310 / 412 ms, 63,432 994 / 393 / 417 ms, 72,242
+// 1,156 / 457 / 503 ms, 100,434 1,034 / 531 / 483 ms, 248,442 1,577 / 1,289 /
+// 788 ms, 495,122 2,026 / 2,551 / 1,535 ms.
 int fp64_rays_per_warp(long long n_rays, int sms) {
+    if (n_rays >= 2LL * kWideRays * kBlocksPerSm * sms) return kWideRays;
     static const double kCost[4] = {226, 205, 190, 175};
     double best = 1e300;
     int R = 1;
     for (int i = 0; i < 4; ++i) {
-        const int r = kMaxRays >> i;
+        const int r = kGroups >> i;
         const double warps = (double)((n_rays + r - 1) / r) / sms;
         const double t = kCost[i] * (warps > 64.0 / 19.0 ? 19.0 * warps : 64.0);
         if (t < best) {
@@ -918,7 +968,8 @@ cudaError_t launch_trace_fp64(const GridDev &g, const FanDev &f, int rays_per_wa
                               cudaStream_t st) {
     const int R = rays_per_warp;
     const long long blocks = (f.n_rays + R - 1) / R;
-    trace_fp64_kernel<<<(unsigned)blocks, 64, fp64_smem_bytes(R), st>>>(g, f, R, out);
+    if (R > kGroups) trace_fp64_kernel<true><<<(unsigned)blocks, 64, fp64_smem_bytes(R), st>>>(g, f, R, out);
+    else trace_fp64_kernel<false><<<(unsigned)blocks, 64, fp64_smem_bytes(R), st>>>(g, f, R, out);
     return cudaGetLastError();
 }
 

@@ -154,9 +154,51 @@ __device__ __forceinline__ void tail64(const RayPhys<double> &rp, const StageIn<
     dy[5] = __dmul_rn(fma(-kprc, dt, fma(H[2], iG, -__dmul_rn(kps, dr))), irs);
 }
 
-// dy/dP' at state y, all in double: Ne and its gradient from the FP64 padded
-// grid (Eq. 13), then the dipole, Appleton-Hartree and Eq. 1.  sth_out
-// receives sin(theta).
+// Polynomials of the one-dimensional weights (Appendix A; Eq. 7 for
+// Catmull-Rom) as Horner coefficients, highest power first: kinds 0 and 1
+// are the weights of nodes j-1 and j, kinds 2 and 3 their derivatives.
+//   kind 0: t p4(t), kind 1: 1 + t^2 p3(t), kind 2: p4(t), kind 3: t p3(t)
+// with p4 of all five coefficients and p3 of the first four.
+static __constant__ double c_poly[2][4][5] = {
+    {{1.0 / 6.0, -5.0 / 12.0, -1.0 / 6.0, 11.0 / 12.0, -0.5},
+     {-0.5, 1.25, 0.5, -2.25, 0.0},
+     {5.0 / 6.0, -5.0 / 3.0, -0.5, 11.0 / 6.0, -0.5},
+     {-2.5, 5.0, 1.5, -4.5, 0.0}},
+    {{0.0, 0.0, -0.5, 1.0, -0.5},
+     {0.0, 0.0, 1.5, -2.5, 0.0},
+     {0.0, 0.0, -1.5, 2.0, -0.5},
+     {0.0, 0.0, 4.5, -5.0, 0.0}}};
+
+// One altitude row's sum, and the same against the derivative weights.
+__device__ __forceinline__ double row64(double u0, double u1, double u2, double u3, const double *w) {
+    return fma(u3, w[3], fma(u2, w[2], fma(u0, w[0], __dmul_rn(u1, w[1]))));
+}
+
+// Weights of one axis at local coordinate t, all four polynomials in one
+// thread: the operations of density64, in its order.
+__device__ __forceinline__ void weights64(const double (*c)[5], double t, double w[4], double d[4]) {
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        const double s = side ? 1.0 - t : t;
+        double p[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            p[k] = fma(s, fma(s, fma(s, c[k][0], c[k][1]), c[k][2]), c[k][3]);
+            if (k == 0 || k == 2) p[k] = fma(s, p[k], c[k][4]);
+        }
+        const double outer = __dmul_rn(p[0], s), inner = __dadd_rn(1.0, __dmul_rn(__dmul_rn(s, s), p[1]));
+        const double dinner = __dmul_rn(s, p[3]);
+        w[side ? 3 : 0] = outer;
+        w[side ? 2 : 1] = inner;
+        d[side ? 3 : 0] = side ? -p[2] : p[2];
+        d[side ? 2 : 1] = side ? -dinner : dinner;
+    }
+}
+
+// dy/dP' at state y, all in double, by one thread: Ne and its gradient from
+// the FP64 padded grid (Eq. 13), then the dipole, Appleton-Hartree and Eq. 1.
+// The same operations in the same order as the lane groups' evaluation.
+// sth_out receives sin(theta).
 __device__ __forceinline__ void rhs64(const GridDev &g, const RayPhys<double> &rp, const double y[6], double dy[6],
                                       double *mu2, double *sth_out = nullptr) {
     StageIn<double> s;
@@ -175,23 +217,31 @@ __device__ __forceinline__ void rhs64(const GridDev &g, const RayPhys<double> &r
     const bool in_b = cell64(grid_coord64(g, 1, y[0], y[1], y[2]), g.n_lon, ib, tb);
     const bool in_c = cell64(grid_coord64(g, 2, y[0], y[1], y[2]), g.n_alt, ic, tc);
     if (in_a && in_b && in_c) {
-        double wa[4], da[4], wb[4], db[4], wc[4], dc[4], out[4];
-        interp_weights<double>(ta, wa, da, g.interp);
-        interp_weights<double>(tb, wb, db, g.interp);
-        interp_weights<double>(tc, wc, dc, g.interp);
+        const double (*c)[5] = c_poly[g.interp == 1 ? 1 : 0];
+        double wa[4], da[4], wb[4], db[4], wc[4], dc[4], out[4] = {0.0, 0.0, 0.0, 0.0};
+        weights64(c, ta, wa, da);
+        weights64(c, tb, wb, db);
+        weights64(c, tc, wc, dc);
         const long long sj = g.p_alt, si = (long long)g.p_lon * g.p_alt;
         // padded index of node (ia-1, ib-1, ic-1) is (ia, ib, ic)
         const double *base = g.pad64 + (long long)ia * si + (long long)ib * sj + ic;
-#define RTGD_ROW64(a, b, u0, u1, u2, u3)              \
-    {                                                 \
-        const double *p_ = base + (a) * si + (b) * sj; \
-        u0 = __ldg(p_);                               \
-        u1 = __ldg(p_ + 1);                           \
-        u2 = __ldg(p_ + 2);                           \
-        u3 = __ldg(p_ + 3);                           \
-    }
-        RTGD_CONTRACT(double, false, RTGD_ROW64, 0.0, 0, 4, wa, da, wb, db, wc, dc, out);
-#undef RTGD_ROW64
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            double sv = 0.0, sd = 0.0, sc = 0.0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const double *p = base + a * si + b * sj;
+                const double u0 = __ldg(p), u1 = __ldg(p + 1), u2 = __ldg(p + 2), u3 = __ldg(p + 3);
+                const double v = row64(u0, u1, u2, u3, wc), dv = row64(u0, u1, u2, u3, dc);
+                sv = fma(v, wb[b], sv);
+                sd = fma(v, db[b], sd);
+                sc = fma(dv, wb[b], sc);
+            }
+            out[0] = fma(sv, wa[a], out[0]);
+            out[1] = fma(sv, da[a], out[1]);
+            out[2] = fma(sd, wa[a], out[2]);
+            out[3] = fma(sc, wa[a], out[3]);
+        }
         s.X = rp.xfac * out[0];
         s.dX[0] = rp.xfac * out[3] * g.inv_dalt;
         s.dX[1] = -rp.xfac * out[1] * g.inv_dlat * kRad2Deg;
