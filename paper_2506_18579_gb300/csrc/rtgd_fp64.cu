@@ -86,9 +86,6 @@ __device__ __forceinline__ bool finite64(double x) {
     return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
 }
 
-// The same with NaN among them: fmax, which ignores a NaN.
-__device__ __noinline__ double max3_rare(double a, double b, double c) { return fmax(fabs(a), fmax(fabs(b), fabs(c))); }
-
 // max of two numbers at least one of which is >= +0 (not NaN): the order of
 // such doubles is the order of their bits as signed integers.
 __device__ __forceinline__ double max_bits(double a, double b) {
@@ -733,8 +730,8 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
                 pos = max_bits(fabs(e0), max_bits(r * fabs(e1), r * sth * fabs(e2)));
                 kerr = max_bits(fabs(e3), max_bits(fabs(e4), fabs(e5)));
             } else {
-                pos = max3_rare(e0, r * e1, r * sth * e2);
-                kerr = max3_rare(e3, e4, e5);
+                pos = max3_rare(e0, r, e1, r * sth, e2);
+                kerr = max3_rare(e3, 1.0, e4, 1.0, e5);
             }
             const double dp = f.atol + f.rtol * r, dk = f.rtol * fmax(kmag, 1e-3);
             double err;

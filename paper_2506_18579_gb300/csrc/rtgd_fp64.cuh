@@ -23,6 +23,13 @@ __device__ __forceinline__ double wrap360(double x) {
     return wrap360_rare(x);
 }
 
+// max(|a|, sb |b|, sc |c|) with infinities or NaN among them: fmax, which
+// ignores a NaN.  A negative scale (sin(theta) beyond a pole) takes its term out
+// of the maximum, as in the step control's bit compare of finite values.
+__host__ __device__ __noinline__ inline double max3_rare(double a, double sb, double b, double sc, double c) {
+    return fmax(fabs(a), fmax(sb * fabs(b), sc * fabs(c)));
+}
+
 // Grid coordinate of a position along one axis (0 latitude, 1 longitude, 2
 // altitude): (90 - deg(theta) - lat0) / dlat, (deg(phi) - lon0 wrapped) / dlon,
 // (r - R_E - alt0) / dalt.  One form for the three axes, chosen by selects, so
