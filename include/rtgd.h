@@ -158,7 +158,8 @@ enum {
     RT_RAY_LEFT_GRID = 3,      /* left the grid sideways inside its altitude span */
     RT_RAY_MAX_STEPS = 4,      /* max_steps attempts used */
     RT_RAY_STEP_UNDERFLOW = 5, /* RKF45 needed a step below h_min_km */
-    RT_RAY_NONFINITE = 6,      /* non-finite state, or mu^2 <= 0 at the transmitter */
+    RT_RAY_NONFINITE = 6,      /* non-finite state, or mu^2 <= 0 at the transmitter (mixed path, grid axis of
+                                  more than 2^20 nodes: also a fixed step across 2^22 cells) */
     RT_RAY_MAX_PATH = 7        /* reached max_group_path_km */
 };
 

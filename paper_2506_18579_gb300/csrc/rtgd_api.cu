@@ -560,6 +560,9 @@ rt_err rt_grid_create(const rt_grid_desc *desc, const void *ne_host, rt_grid **o
     d.mf[2] = (float)d.m[2];
     d.top_f = (float)d.top;
     d.alt0_f = (float)d.alt0;
+    const bool long_axis = std::max(desc->n_lat, std::max(desc->n_lon, desc->n_alt)) > (1 << 20);
+    d.far_cells = long_axis ? 1 << 30 : 1 << 21;
+    d.far_stage = long_axis ? 4194303.0f : INFINITY;
     d.iso = d.b0 == 0.0 ? 1 : 0;
     d.interp = (desc->flags & RT_GRID_CATMULL_ROM) ? 1 : 0;
     d.pad64 = g->pad64;

@@ -38,6 +38,12 @@ struct GridDev {
     float sa, sb, sc;                // d(grid coord)/d(theta, phi, r): -rad2deg/dlat, rad2deg/dlon, 1/dalt
     float R_Ef, mf[3];               // float copies of R_E and m
     float top_f, alt0_f;             // top and alt0 as floats
+    // Mixed path: base cells are kept within +-far_cells, and a stage offset of
+    // more than far_stage cells makes its derivatives NaN.  2^21 and no limit; on
+    // an axis of more than 2^20 nodes 2^30 (no axis has more: 4 nodes on each of
+    // the others, 2^34 in all) and the offsets that stage_cell resolves.
+    int far_cells;
+    float far_stage;
     int iso;                         // no field (b0 == 0)
     int interp;                      // 0: Galerkin-Difference p=3, 1: Catmull-Rom (comparison)
     const double *pad64;             // (n_lat+2)(n_lon+2)(n_alt+2) doubles

@@ -225,22 +225,22 @@ __device__ __forceinline__ float narrow(double x) {
     return __uint_as_float((unsigned)(r >> 29) | ((unsigned)(b >> 32) & 0x80000000u));
 }
 
-__device__ __noinline__ int floor_cell_rare(double x, float *t) {
+__device__ __noinline__ int floor_cell_rare(double x, float *t, int far) {
     const double f = floor(x);
     *t = (float)(x - f);
-    return (int)fmin(fmax(f, -1e6), 1e6);
+    return (int)fmin(fmax(f, -(double)far), (double)far);
 }
 
 // floor(x) as an integer and the fraction x - floor(x): one addition rounded
-// down.  Beyond +-10^6 (and for NaN) the cell is clamped to that (negative
-// side for NaN), which stays outside of the grid.
-__device__ __forceinline__ int floor_cell(double x, float &t) {
+// down.  Beyond +-far (and for NaN) the cell is clamped to that (negative side
+// for NaN), which lies outside of the grid.
+__device__ __forceinline__ int floor_cell(double x, float &t, int far) {
     const double magic = 6755399441055744.0;  // 1.5 * 2^52
     const int hi = __double2hiint(x) & 0x7fffffff;
-    if (hi >= 0x412e8480) return floor_cell_rare(x, &t);  // |x| >= 10^6
+    if (hi >= 0x41d00000) return floor_cell_rare(x, &t, far);  // |x| >= 2^30
     const double big = __dadd_rd(x, magic);
     t = narrow(x - (big - magic));
-    return __double2loint(big);
+    return min(max(__double2loint(big), -far), far);
 }
 
 // Base of a double state (double arithmetic; used at launch and to resync).
@@ -251,14 +251,15 @@ __device__ __forceinline__ int floor_cell(double x, float &t) {
 // 8 in lane_fold), where floors, clamps, conversions and a division-free wrap
 // in FP64 made it ~65.
 __device__ __noinline__ Base32 base_of(double lat0, double lon0, double inv_dlat, double inv_dlon, double R_E,
-                                       double alt0, double inv_dalt, double r, double th, double ph) {
+                                       double alt0, double inv_dalt, int far, double r, double th,
+                                       double ph) {
     Base32 b;
     const double lat = 90.0 - th * kRad2Deg;
     const double lonrel = wrap360(ph * kRad2Deg - lon0);
     const double alt = r - R_E;
-    b.ia = floor_cell((lat - lat0) * inv_dlat, b.ta);
-    b.ib = floor_cell(lonrel * inv_dlon, b.tb);
-    b.ic = floor_cell((alt - alt0) * inv_dalt, b.tc);
+    b.ia = floor_cell((lat - lat0) * inv_dlat, b.ta, far);
+    b.ib = floor_cell(lonrel * inv_dlon, b.tb, far);
+    b.ic = floor_cell((alt - alt0) * inv_dalt, b.tc, far);
     b.r = narrow(r);
     b.alt = narrow(alt);
     sincosf(narrow(th), &b.sth, &b.cth);
@@ -267,15 +268,16 @@ __device__ __noinline__ Base32 base_of(double lat0, double lon0, double inv_dlat
 }
 
 __device__ __forceinline__ void base_from_state(const GridDev &g, const double y[6], Base32 &b) {
-    b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, y[0], y[1], y[2]);
+    b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, g.far_cells, y[0], y[1], y[2]);
 #pragma unroll
     for (int i = 0; i < 3; ++i) b.k[i] = (float)y[3 + i];
 }
 
+// (A shift of more than 2^29 cells stays in t; the index stays within 1.5 * 2^30.)
 __device__ __forceinline__ void shift_axis(int &i, float &t, float dt) {
     const float u = t + dt;
-    const float fl = fminf(fmaxf(floorf(u), -1e6f), 1e6f);
-    i += (int)fl;
+    const float fl = fminf(fmaxf(floorf(u), -0x1p29f), 0x1p29f);
+    i = min(max(i, -(1 << 30)), 1 << 30) + (int)fl;
     t = u - fl;
 }
 
@@ -322,10 +324,10 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float d) {
 // delta * scale; false outside [0, n-1], and then cell 0 at t = 0, so that the
 // caller can gather from an in-bounds cell without branching.  On the critical
 // path of every stage, so floor(t) costs one addition: t + 1.5 * 2^23 rounded
-// down holds it in the low mantissa bits.  That is exact for |t| < 2^22; beyond
+// down holds it in the low mantissa bits.  That is exact for |t| < 2^22.  Beyond
 // that, and for NaN, the integer lands at least 2^22 cells out, which the index
-// test refuses (base cells lie within +-10^6 of the grid, grids have fewer
-// nodes per axis than that).  Nine instructions; with a clamp and a
+// test refuses where base cells lie within 2^21 of a grid of at most 2^20 nodes
+// per axis; longer axes have g.far_stage.  Nine instructions; with a clamp and a
 // round-to-nearest that was corrected afterwards it took sixteen.
 __device__ __forceinline__ bool stage_cell(int i0, float t, int n, int &i, float &tt) {
     const float magic = 12582912.0f;
@@ -383,7 +385,10 @@ template <int STENCIL, int G, int IP, bool FIRST = false>
 __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float> &rp, const Base32 &b,
                                           const float d[6], float dy[6], float *mu2, int q, unsigned gmask) {
     StageIn<float> s;
-    s.r = b.r + d[0];
+    const float xa = b.ta + g.sa * d[1], xb = b.tb + g.sb * d[2], xc = b.tc + g.sc * d[0];
+    // beyond far_stage NaN, so that the adaptive step control retries with a
+    // smaller step and a fixed step ends the ray as not finite
+    s.r = fmaxf(fmaxf(fabsf(xa), fabsf(xb)), fabsf(xc)) <= g.far_stage ? b.r + d[0] : NAN;
     angle_add(b.sth, b.cth, d[1], s.sth, s.cth);
     angle_add(b.sph, b.cph, d[2], s.sph, s.cph);
     s.k[0] = b.k[0] + d[3];
@@ -392,9 +397,9 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
     const FieldTerms<float> F = field_terms<float>(rp, s);
     int ia, ib, ic;
     float ta, tb, tc;
-    const bool in_a = stage_cell(b.ia, b.ta + g.sa * d[1], g.n_lat, ia, ta);
-    const bool in_b = stage_cell(b.ib, b.tb + g.sb * d[2], g.n_lon, ib, tb);
-    const bool in_c = stage_cell(b.ic, b.tc + g.sc * d[0], g.n_alt, ic, tc);
+    const bool in_a = stage_cell(b.ia, xa, g.n_lat, ia, ta);
+    const bool in_b = stage_cell(b.ib, xb, g.n_lon, ib, tb);
+    const bool in_c = stage_cell(b.ic, xc, g.n_alt, ic, tc);
     const bool inside = in_a & in_b & in_c;  // each axis is in bounds by itself
     float wa[4], da[4], wb[4], db[4], wc[4], dc[4], out[4], ref;
     constexpr int NA = 4 / G;
@@ -612,7 +617,7 @@ __device__ __forceinline__ void accumulate_next(Lane &L, const Tableau &T, int s
 // Base of the transmitter position (the launch state of every ray of the
 // fan; the wave vector part is set per ray).
 __device__ __forceinline__ Base32 tx_base(const GridDev &g, const FanDev &f) {
-    Base32 b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, f.tx_r, f.tx_th, f.tx_ph);
+    Base32 b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, g.far_cells, f.tx_r, f.tx_th, f.tx_ph);
     b.k[0] = b.k[1] = b.k[2] = 0.0f;
     return b;
 }
@@ -1002,7 +1007,7 @@ __device__ bool lane_end_attempt(Lane &L, const GridDev &g, const FanDev &f, Lan
     if (++L.since_sync >= kResyncSteps) {
         L.since_sync = 0;
         lane_fold(L);
-        L.b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, L.y[0], L.y[1], L.y[2]);
+        L.b = base_of(g.lat0, g.lon0, g.inv_dlat, g.inv_dlon, g.R_E, g.alt0, g.inv_dalt, g.far_cells, L.y[0], L.y[1], L.y[2]);
 #pragma unroll
         for (int i = 0; i < 3; ++i) L.b.k[i] = L.k_hi[i] + L.k_lo[i];
     } else {
