@@ -45,35 +45,36 @@ FLOP_PER_EVAL = {"mixed": 1000.0, "fp64": 910.0}
 GATHER_BYTES = {"mixed": 65 * 4, "fp64": 64 * 8}
 # DRAM bytes (read + write) of one launch of the benchmark's dominant kernel,
 # from an ncu capture of the same launch (cold caches, as after the
-# L2 flush between timed steps), keyed by workload and launch configuration
-# (kernel, stencil, lanes per ray) and valid only for the kernel sources it
-# was captured from: a changed kernel reports traffic null.
-KERNEL_SOURCES = tuple("paper_2506_18579_gb300/csrc/" + f for f in (
-    "rtgd_kernels.cu", "rtgd_device.cuh", "rtgd_fan.cuh", "rtgd_fp64.cuh"))
+# L2 flush between timed steps), keyed by workload, precision and launch
+# configuration (kernel, stencil, lanes per ray) and valid only for the kernel
+# sources it was captured from: a changed kernel reports traffic null.
+KERNEL_SOURCES = {p: tuple("paper_2506_18579_gb300/csrc/" + f for f in files) for p, files in {
+    "mixed": ("rtgd_kernels.cu", "rtgd_device.cuh", "rtgd_fan.cuh", "rtgd_fp64.cuh"),
+    "fp64": ("rtgd_fp64.cu", "rtgd_fp64.cuh", "rtgd_fan.cuh", "rtgd_device.cuh")}.items()}
 TRAFFIC = {
-    # key = (workload, kernel, stencil, lanes per ray); the anisotropic fan in
-    # the autotuner's configurations (plain, 4 lanes, 96-thread blocks)
-    ("c2", 1, 3, 4): {"bytes_per_launch": 27159040 + 85504, "source_sha256": "fa834026b2b0187e"},
-    ("c2", 1, 2, 4): {"bytes_per_launch": 5581824 + 27904, "source_sha256": "fa834026b2b0187e"},
+    # key = (workload, precision, kernel, stencil, lanes per ray); the anisotropic
+    # fan in the autotuner's configurations (plain, 4 lanes, 96-thread blocks)
+    ("c2", "mixed", 1, 3, 4): {"bytes_per_launch": 27159040 + 85504, "source_sha256": "fa834026b2b0187e"},
+    ("c2", "mixed", 1, 2, 4): {"bytes_per_launch": 5581824 + 27904, "source_sha256": "fa834026b2b0187e"},
     # the ionogram batch, one lane per ray (the only lane count the autotuner
     # tries on a fan this large): plain kernel with 32-thread blocks (table
     # and quad stencils), persistent kernel with 128-thread blocks
-    ("c4", 1, 3, 1): {"bytes_per_launch": 20942848 + 2286080, "source_sha256": "fa834026b2b0187e"},
-    ("c4", 1, 2, 1): {"bytes_per_launch": 4317952 + 1300224, "source_sha256": "fa834026b2b0187e"},
-    ("c4", 2, 3, 1): {"bytes_per_launch": 20998144 + 1057792, "source_sha256": "fa834026b2b0187e"},
+    ("c4", "mixed", 1, 3, 1): {"bytes_per_launch": 20942848 + 2286080, "source_sha256": "fa834026b2b0187e"},
+    ("c4", "mixed", 1, 2, 1): {"bytes_per_launch": 4317952 + 1300224, "source_sha256": "fa834026b2b0187e"},
+    ("c4", "mixed", 2, 3, 1): {"bytes_per_launch": 20998144 + 1057792, "source_sha256": "fa834026b2b0187e"},
 }
 SMS = 152
 FP32_LANES_PER_SM = 128
 FP64_FMA_PER_SM_CLK = 2  # GB300: FP64 issue rate is 1/64 of FP32
 
 
-def kernel_source_hash():
-    """Hash of the kernel code (comments and whitespace removed, so that a
+def kernel_source_hash(precision="mixed"):
+    """Hash of the code of the path's kernel (comments and whitespace removed, so that a
     comment edit does not invalidate a capture)."""
     import hashlib
     import re
     h = hashlib.sha256()
-    for rel in KERNEL_SOURCES:
+    for rel in KERNEL_SOURCES[precision]:
         with open(os.path.join(ROOT, rel), encoding="utf-8") as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)  # block comments
@@ -82,12 +83,12 @@ def kernel_source_hash():
     return h.hexdigest()[:16]
 
 
-def captured_traffic(workload, cfg):
+def captured_traffic(workload, cfg, precision="mixed"):
     """DRAM bytes per launch from the capture of this exact kernel, or None."""
     if cfg is None:
         return None
-    rec = TRAFFIC.get((workload, int(cfg.kernel), int(cfg.stencil), int(cfg.lanes_per_ray)))
-    if rec is None or rec["source_sha256"] != kernel_source_hash():
+    rec = TRAFFIC.get((workload, precision, int(cfg.kernel), int(cfg.stencil), int(cfg.lanes_per_ray)))
+    if rec is None or rec["source_sha256"] != kernel_source_hash(precision):
         return None
     return rec["bytes_per_launch"]
 
@@ -609,9 +610,9 @@ def run_ours(args):
             "tighter_rtol": nominal,
             "fp64_gpu_path": {"rays_per_s": n / fp64_s, "seconds": fp64_s, "critical_path": fp64_alone},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                         "frac": achieved / peak, "traffic": captured_traffic(args.workload, cfg),
+                         "frac": achieved / peak, "traffic": captured_traffic(args.workload, cfg, args.precision),
                          "traffic_unit": "bytes per launch (DRAM read + write, ncu)",
-                         "kernel_source_sha256": kernel_source_hash(), "peak_basis": bound_note,
+                         "kernel_source_sha256": kernel_source_hash(args.precision), "peak_basis": bound_note,
                          "flop_per_stage_eval": FLOP_PER_EVAL[args.precision],
                          "measured_peaks": peaks,
                          "frac_of_measured": achieved / (peaks["fp32_fma_tflops"] if prec == rt.RT_MIXED
