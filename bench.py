@@ -5,7 +5,10 @@ One step = one fan of the anisotropic workload (E + F2 + TID ionosphere on a
 91x181x151 FP32 grid, centred dipole, 8/12/16 MHz x 115 elevations x 36
 azimuths x O/X = 24,840 rays, RKF45 at rtol 1e-8) traced through the C ABI.
 The grid is resident on the device (created once, as in serving); inputs of a
-step are the fan arrays.  Prints one JSON line (rank 0).
+step are the fan arrays.  Prints one JSON line (rank 0): the headline
+figures, short enough for a reader that keeps only the end of the output.
+Everything measured besides (accuracy by output, batch, serving, critical
+paths) is one JSON line on the error output, after "details ".
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--precision mixed|fp64]
                   [--impl ours|reference]
@@ -91,6 +94,35 @@ def captured_traffic(workload, cfg, precision="mixed"):
     if rec is None or rec["source_sha256"] != kernel_source_hash(precision):
         return None
     return rec["bytes_per_launch"]
+
+
+# The headline line's keys; a dict names the entries kept of a nested record.
+HEADLINE = {
+    **dict.fromkeys(("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+                     "scaling", "vs_baseline", "dtype", "data", "config", "ray_steps_per_s", "fan_latency_ms", "e2e",
+                     "gpu_launches")),
+    "clocks": ("sm_mhz", "sm_max_mhz", "reasons"),
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "traffic"),
+    "cpu_baseline": ("value", "unit", "cores", "kind"),
+}
+HEADLINE_CHARS = 1400  # at most
+
+
+def headline(line):
+    """The headline part of a full result line, numbers to seven digits."""
+    def short(v):
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return float("%.7g" % v) if isinstance(v, float) else v
+    out = {}
+    for k, keep in HEADLINE.items():
+        v = line[k]
+        out[k] = short({e: v[e] for e in keep} if keep and v is not None else v)
+    acc = line["accuracy"].get("vs_cpu_oracle")
+    if acc is not None:
+        out["accuracy"] = short({e: acc[e] for e in ("rays_compared", "status_mismatch", "p_and_d_within_bar_share")
+                                 if e in acc})
+    return out
 
 
 def parse_args():
@@ -637,7 +669,8 @@ def run_ours(args):
         }
     grid.close()
     if line is not None:
-        print(json.dumps(line), flush=True)
+        print("details " + json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
 
