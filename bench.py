@@ -66,6 +66,7 @@ TRAFFIC = {
     ("c4", "mixed", 1, 2, 1): {"bytes_per_launch": 4317952 + 1300224, "source_sha256": "fa834026b2b0187e"},
     ("c4", "mixed", 2, 3, 1): {"bytes_per_launch": 20998144 + 1057792, "source_sha256": "fa834026b2b0187e"},
 }
+LAUNCHES_PER_STEP = 2  # the trace kernel and the pass that finishes the records, in both precisions
 SMS = 152
 FP32_LANES_PER_SM = 128
 FP64_FMA_PER_SM_CLK = 2  # GB300: FP64 issue rate is 1/64 of FP32
@@ -580,8 +581,8 @@ def run_ours(args):
         alone_ms, _ = time_one_ray(rt, torch, grid, one_ray_spec(wl, spec, i_long), prec, cfg, 3, 2)
         critical = {"longest_ray_alone_ms": alone_ms, "fan_ms": mean_ms, "fan_over_alone": mean_ms / alone_ms,
                     "ns_per_stage_eval_alone": alone_ms * 1e6 / max(int(res["n_evals"][i_long]), 1)}
-        # the FP64 path's own critical path: its longest ray traced alone (one
-        # thread per ray), beside its whole-fan time
+        # the FP64 path's own critical path: its longest ray traced alone, beside
+        # its whole-fan time
         fp64_alone = None
         if prec == rt.RT_MIXED:
             i64 = int(np.argmax(ref64["n_evals"]))
@@ -659,7 +660,7 @@ def run_ours(args):
             "cpu_baseline": cpu,
             "e2e": {"value": n * world / e2e_s, "unit": "rays/s", "h2d_bytes_per_step": fan.host_bytes,
                     "d2h_bytes_per_step": n * 64},
-            "gpu_launches": args.steps * (2 if prec == rt.RT_MIXED else 1),  # trace (+ finish pass) per step
+            "gpu_launches": args.steps * LAUNCHES_PER_STEP,
             "clocks": clk,
             "wall_s_timed": t_wall,
             "tune_ms": tune_ms,
