@@ -1286,8 +1286,10 @@ rt_err rt_eval_rhs(const rt_grid *grid, double freq_mhz, int32_t mode, int32_t p
     CUDA_TRY(cudaMalloc((void **)&buf, n * 13 * sizeof(double)));
     cudaError_t e = cudaMemcpy(buf, y_host, n * 6 * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = launch_eval_rhs(grid->g, buf, buf + n * 6, buf + n * 12, freq_mhz, mode, precision, stencil,
-                            (long long)n, nullptr);
+        e = precision == RT_FP64 ? launch_eval_rhs_fp64(grid->g, buf, buf + n * 6, buf + n * 12, freq_mhz, mode,
+                                                        props(grid->device).sms, (long long)n, nullptr)
+                                 : launch_eval_rhs(grid->g, buf, buf + n * 6, buf + n * 12, freq_mhz, mode, stencil,
+                                                   (long long)n, nullptr);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMemcpy(dy_host, buf + n * 6, n * 6 * sizeof(double), cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(mu2_host, buf + n * 12, n * sizeof(double), cudaMemcpyDeviceToHost);

@@ -923,6 +923,72 @@ __global__ void __launch_bounds__(64, kBlocksPerSm) trace_fp64_kernel(const __gr
     duo.start(0, lane);  // the helper ends
 }
 
+// dy/dP' at the states of a block (diagnostic): G lanes each, as run_rays
+// evaluates k1; count of them, in the slots.
+template <int G>
+__device__ __forceinline__ void eval_states(const GridDev &g, int mode, double *slots, double *scratch, int count,
+                                            double *__restrict__ dys, Duo &duo) {
+    const int lane = threadIdx.x, grp = lane / G, q = lane % G;
+    const bool has = grp < count;
+    double *S = slots + (has ? grp : 0) * kSlot;
+    double *C = scratch + grp * (G == 1 ? cLane : cGroup);
+    RayPhys<double> rp;
+    rp.xfac = S[kXfac];
+    rp.ab0 = S[kAb0];
+    rp.R_E = g.R_E;
+    rp.m[0] = g.m[0];
+    rp.m[1] = g.m[1];
+    rp.m[2] = g.m[2];
+    rp.iso = g.iso != 0;
+    rp.mode = mode;
+    if (G > 1 && q == 0) duo.slot_of[grp] = has ? grp : 0;
+    if (G == 32 && q == 0) duo.D[Duo::dXfac] = rp.xfac;
+    __syncwarp();
+    stage64<G>(g, rp, S + kY, true, C, q, S + kK1, has, duo);
+    __syncwarp();
+    for (int c = q; has && c < 6; c += G) dys[grp * 6 + c] = S[kK1 + c];
+}
+
+// R states per block, as many as a warp of a trace of n rays starts with: so the
+// states are evaluated by the same code as that trace's, 1, 4, 8, 16 or 32 lanes
+// each.  mu^2 is the launch's evaluation.
+__global__ void __launch_bounds__(64, kBlocksPerSm) eval_rhs_fp64_kernel(const __grid_constant__ GridDev g,
+                                                                      const double *__restrict__ ys,
+                                                                      double *__restrict__ dys,
+                                                                      double *__restrict__ mu2s, double f_hz, int mode,
+                                                                      int R, long long n) {
+    extern __shared__ double sm[];
+    double *coef = sm, *hand = coef + kPoly + kPow2, *slots = hand + Duo::dSize, *scratch = slots + R * kSlot;
+    int *map = (int *)(scratch + fp64_scratch(R));
+    Duo duo{hand, map + R, map + R + 1, sm};
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x >= 32) {
+        helper64(g, slots, scratch, coef, lane, duo);
+        return;
+    }
+    if (lane < kPoly) coef[lane] = (&c_poly[g.interp == 1 ? 1 : 0][0][0])[lane];
+    const long long first = (long long)blockIdx.x * R;
+    const int count = (int)(n - first < R ? n - first : R);
+    if (lane < count) {
+        const RayPhys<double> rp = make_phys<double>(g, f_hz, mode);
+        double *S = slots + lane * kSlot;
+        double y[6], dy[6], mu2;
+        for (int c = 0; c < 6; ++c) S[kY + c] = y[c] = ys[(first + lane) * 6 + c];
+        S[kXfac] = rp.xfac;
+        S[kAb0] = rp.ab0;
+        rhs64(g, rp, y, dy, &mu2);
+        mu2s[first + lane] = mu2;
+    }
+    __syncwarp();
+    dys += first * 6;
+    if (R > kGroups) eval_states<1>(g, mode, slots, scratch, count, dys, duo);
+    else if (R > 4) eval_states<4>(g, mode, slots, scratch, count, dys, duo);
+    else if (R > 2) eval_states<8>(g, mode, slots, scratch, count, dys, duo);
+    else if (R > 1) eval_states<16>(g, mode, slots, scratch, count, dys, duo);
+    else eval_states<32>(g, mode, slots, scratch, count, dys, duo);
+    duo.start(0, lane);  // the helper ends
+}
+
 }  // namespace
 
 // Rays a warp starts with, by the rays per SM.  One while the first warps, one
@@ -958,6 +1024,15 @@ cudaError_t launch_trace_fp64(const GridDev &g, const FanDev &f, int rays_per_wa
     const long long blocks = (f.n_rays + R - 1) / R;
     if (R > kGroups) trace_fp64_kernel<true><<<(unsigned)blocks, 64, fp64_smem_bytes(R), st>>>(g, f, R, out);
     else trace_fp64_kernel<false><<<(unsigned)blocks, 64, fp64_smem_bytes(R), st>>>(g, f, R, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_eval_rhs_fp64(const GridDev &g, const double *ys, double *dys, double *mu2s, double freq_mhz,
+                                 int mode, int sms, long long n, cudaStream_t st) {
+    if (n == 0) return cudaSuccess;
+    const int R = fp64_rays_per_warp(n, sms);
+    eval_rhs_fp64_kernel<<<(unsigned)((n + R - 1) / R), 64, fp64_smem_bytes(R), st>>>(g, ys, dys, mu2s, freq_mhz * 1e6,
+                                                                                     mode, R, n);
     return cudaGetLastError();
 }
 

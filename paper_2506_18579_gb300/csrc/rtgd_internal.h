@@ -129,7 +129,11 @@ constexpr int kNoallocMaxTable = 4096;
 constexpr size_t kNoallocScratchBytes = 16 + 3 * (size_t)kNoallocMaxTable * sizeof(double);
 cudaError_t noalloc_scratch(int device, void **ptr, size_t *bytes);
 
+// dy/dP' and mu^2 at n states, mixed and FP64 (there with the lanes per state
+// that a trace of n rays starts with on a device with sms SMs).
 cudaError_t launch_eval_rhs(const GridDev &g, const double *ys, double *dys, double *mu2s, double freq_mhz, int mode,
-                            int precision, int stencil, long long n, cudaStream_t st);
+                            int stencil, long long n, cudaStream_t st);
+cudaError_t launch_eval_rhs_fp64(const GridDev &g, const double *ys, double *dys, double *mu2s, double freq_mhz,
+                                 int mode, int sms, long long n, cudaStream_t st);
 
 }  // namespace rtgd

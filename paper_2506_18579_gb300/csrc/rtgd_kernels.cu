@@ -1254,38 +1254,30 @@ cudaError_t launch_ionogram(const rt_ray_result *res, const double *freq, const 
 }
 
 // ============================================================== diagnostics
+// The mixed path's right-hand side (the FP64 path's: eval_rhs_fp64_kernel).
 __global__ void eval_rhs_kernel(GridDev g, const double *__restrict__ ys, double *__restrict__ dys,
-                                double *__restrict__ mu2s, double freq_mhz, int mode, int precision, int stencil,
-                                long long n) {
+                                double *__restrict__ mu2s, double freq_mhz, int mode, int stencil, long long n) {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double y[6], dy[6], mu2 = 0.0;
+    double y[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) y[c] = ys[i * 6 + c];
-    if (precision == RT_FP64) {
-        const RayPhys<double> rp = make_phys<double>(g, freq_mhz * 1e6, mode);
-        rhs64(g, rp, y, dy, &mu2);
+    const RayPhys<float> rp = make_phys<float>(g, freq_mhz * 1e6, mode);
+    Base32 b;
+    base_from_state(g, y, b);
+    float d[6] = {0, 0, 0, 0, 0, 0}, dyf[6], m2;
+    if (g.interp == 1) {
+        if (stencil == RT_STENCIL_TABLE) rhs_mixed<RT_STENCIL_TABLE, 1, 1>(g, rp, b, d, dyf, &m2, 0, 0u);
+        else if (stencil == RT_STENCIL_GATHER) rhs_mixed<RT_STENCIL_GATHER, 1, 1>(g, rp, b, d, dyf, &m2, 0, 0u);
+        else rhs_mixed<RT_STENCIL_QUAD, 1, 1>(g, rp, b, d, dyf, &m2, 0, 0u);
     } else {
-        const RayPhys<float> rp = make_phys<float>(g, freq_mhz * 1e6, mode);
-        Base32 b;
-        base_from_state(g, y, b);
-        float d[6] = {0, 0, 0, 0, 0, 0}, dyf[6], m2;
-        if (g.interp == 1) {
-            if (stencil == RT_STENCIL_TABLE) rhs_mixed<RT_STENCIL_TABLE, 1, 1>(g, rp, b, d, dyf, &m2, 0, 0u);
-            else if (stencil == RT_STENCIL_GATHER) rhs_mixed<RT_STENCIL_GATHER, 1, 1>(g, rp, b, d, dyf, &m2, 0, 0u);
-            else rhs_mixed<RT_STENCIL_QUAD, 1, 1>(g, rp, b, d, dyf, &m2, 0, 0u);
-        } else {
-            if (stencil == RT_STENCIL_TABLE) rhs_mixed<RT_STENCIL_TABLE, 1, 0>(g, rp, b, d, dyf, &m2, 0, 0u);
-            else if (stencil == RT_STENCIL_GATHER) rhs_mixed<RT_STENCIL_GATHER, 1, 0>(g, rp, b, d, dyf, &m2, 0, 0u);
-            else rhs_mixed<RT_STENCIL_QUAD, 1, 0>(g, rp, b, d, dyf, &m2, 0, 0u);
-        }
-#pragma unroll
-        for (int c = 0; c < 6; ++c) dy[c] = dyf[c];
-        mu2 = m2;
+        if (stencil == RT_STENCIL_TABLE) rhs_mixed<RT_STENCIL_TABLE, 1, 0>(g, rp, b, d, dyf, &m2, 0, 0u);
+        else if (stencil == RT_STENCIL_GATHER) rhs_mixed<RT_STENCIL_GATHER, 1, 0>(g, rp, b, d, dyf, &m2, 0, 0u);
+        else rhs_mixed<RT_STENCIL_QUAD, 1, 0>(g, rp, b, d, dyf, &m2, 0, 0u);
     }
 #pragma unroll
-    for (int c = 0; c < 6; ++c) dys[i * 6 + c] = dy[c];
-    mu2s[i] = mu2;
+    for (int c = 0; c < 6; ++c) dys[i * 6 + c] = dyf[c];
+    mu2s[i] = m2;
 }
 
 // ================================================================ launchers
@@ -1518,11 +1510,11 @@ cudaError_t persistent_occupancy(int stencil, int lanes, int threads, int *block
 }
 
 cudaError_t launch_eval_rhs(const GridDev &g, const double *ys, double *dys, double *mu2s, double freq_mhz, int mode,
-                            int precision, int stencil, long long n, cudaStream_t st) {
+                            int stencil, long long n, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     const int threads = 128;
     eval_rhs_kernel<<<(unsigned)((n + threads - 1) / threads), threads, 0, st>>>(g, ys, dys, mu2s, freq_mhz, mode,
-                                                                               precision, stencil, n);
+                                                                               stencil, n);
     return cudaGetLastError();
 }
 
