@@ -724,7 +724,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
         if (adaptive) {
             const double r = S[kY], sth = S[kSth], ky = S[kY + 3], kt = S[kY + 4], kp = S[kY + 5];
             const double e0 = C[cE], e1 = C[cE + 1], e2 = C[cE + 2], e3 = C[cE + 3], e4 = C[cE + 4], e5 = C[cE + 5];
-            const double kmag = sqrt(ky * ky + kt * kt + kp * kp);
+            const double kmag = sqrt(fma(kp, kp, fma(ky, ky, __dmul_rn(kt, kt))));
             double pos, kerr;
             if (finite64(e0) && finite64(e1) && finite64(e2) && finite64(e3) && finite64(e4) && finite64(e5)) {
                 pos = max_bits(fabs(e0), max_bits(r * fabs(e1), r * sth * fabs(e2)));
@@ -733,7 +733,7 @@ __device__ __forceinline__ void run_rays(const GridDev &g, const FanDev &f, doub
                 pos = max3_rare(e0, r, e1, r * sth, e2);
                 kerr = max3_rare(e3, 1.0, e4, 1.0, e5);
             }
-            const double dp = f.atol + f.rtol * r, dk = f.rtol * fmax(kmag, 1e-3);
+            const double dp = fma(f.rtol, r, f.atol), dk = f.rtol * fmax(kmag, 1e-3);
             double err;
             if constexpr (G == 1) {
                 err = fmax(pos / dp, kerr / dk);
