@@ -254,14 +254,13 @@ __device__ __forceinline__ RayPhys<R> make_phys(const GridDev &g, double f_hz, i
 // S = sqrt(T^2 + 4 L u^2)) is rewritten with S - T = 4 L u^2 / (S + T), which
 // gives mu^2 = 1 - X / (1 + g), g = 2 L u / (S + T): the same function, free
 // of the 0/0 at X = 1.  Extraordinary wave: the printed form.
-// FIRST spells out which product of S's sum is fused (the first); otherwise the
-// compiler's choice, which has gone either way with the code around it.
-__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
-template <typename R, bool FIRST = false>
+// FIRST: which product of S's sum is fused, T^2 or (4 L u) u.  Spelt out because
+// the compiler's choice has gone either way with the code around it, and the
+// records must not: each kernel states the form its records have.
+template <typename R, bool FIRST>
 __device__ __forceinline__ void appleton_hartree(R X, R L, R T, int mode, R &mu2, R &FX, R &FL, R &FT) {
     const R u = R(1) - X;
-    const R S = fsqrt(FIRST ? fma_rn(T, T, R(4) * L * u * u) : T * T + R(4) * L * u * u);
+    const R S = fsqrt(FIRST ? __fmaf_rn(T, T, R(4) * L * u * u) : __fmaf_rn(R(4) * L * u, u, T * T));
     if (mode > 0) {
         // one reciprocal gives 1/S, 1/W and 1/(1 + g) = W/V with V = W + 2 L u
         const R W = S + T;
@@ -352,7 +351,7 @@ __device__ __forceinline__ FieldTerms<R> field_terms(const RayPhys<R> &rp, const
 //   dk_th/dP'  = (H_th/G - k_th dr + k_ph r cos dphi) / r,
 //   dk_ph/dP'  = (H_ph/G - k_ph sin dr - k_ph r cos dtheta) / (r sin).
 // F holds the field terms of the same stage; mu2_out receives mu^2.
-template <typename R, bool FIRST = false>
+template <typename R, bool FIRST>
 __device__ __forceinline__ void ray_rhs(const RayPhys<R> &rp, const StageIn<R> &s, const FieldTerms<R> &F, R dy[6],
                                         R *mu2_out) {
     const R kr = s.k[0], kt = s.k[1], kp = s.k[2];

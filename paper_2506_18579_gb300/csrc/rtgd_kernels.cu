@@ -381,7 +381,7 @@ __device__ __forceinline__ unsigned long long row_index(int i, int n_j, int j, i
 // so all lanes hold bitwise equal results.  The body has no branch: the field
 // terms (which do not need Ne) come first and can overlap the sample gathers,
 // and a stage outside the grid gathers from cell 0 and discards the result.
-template <int STENCIL, int G, int IP, bool FIRST = false>
+template <int STENCIL, int G, int IP, bool FIRST>
 __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float> &rp, const Base32 &b,
                                           const float d[6], float dy[6], float *mu2, int q, unsigned gmask) {
     StageIn<float> s;
@@ -777,7 +777,7 @@ __device__ __forceinline__ bool lane_next_attempt(Lane &L, const FanDev &f) {
 
 // The launch evaluation: mu^2 at the transmitter for the launch direction,
 // then |k| = mu.  Returns true when the ray has finished (status set).
-template <int STENCIL, int G, int IP, bool FIRST = false>
+template <int STENCIL, int G, int IP, bool FIRST>
 __device__ bool lane_launch(Lane &L, const GridDev &g, const FanDev &f, int q, unsigned gmask) {
     const RayPhys<float> rp = lane_phys(g, L);
     float d[6], ks[6], mu2;
@@ -828,7 +828,7 @@ __device__ __forceinline__ void lane_stage0_done(Lane &L, const GridDev &g, cons
 // stage evaluation serves all stages, which keeps the loop inside the
 // instruction cache; with 2 or 4 lanes per ray (latency-bound fans) stage 0
 // is a separate copy, which schedules better.
-template <int STENCIL, int G, int IP, bool FIRST = false>
+template <int STENCIL, int G, int IP, bool FIRST>
 __device__ __forceinline__ void lane_attempt(Lane &L, const GridDev &g, const FanDev &f, const Tableau &T, int q,
                                              unsigned gmask) {
     const RayPhys<float> rp = lane_phys(g, L);
@@ -1058,6 +1058,7 @@ __device__ __forceinline__ unsigned group_mask(int lane) {
 // warp's stage evaluation faster.
 template <int STENCIL, int G, int IP>
 __global__ void __launch_bounds__(128, G == 1 ? 3 : 2) trace_mixed_plain_kernel(GridDev g, FanDev f, rt_ray_result *__restrict__ out) {
+    constexpr bool FIRST = G > 1;  // see appleton_hartree
     __shared__ Tableau T;
     __shared__ Base32 btx;
     load_tableau(T, f.integrator, &btx, &g, &f);
@@ -1071,7 +1072,7 @@ __global__ void __launch_bounds__(128, G == 1 ? 3 : 2) trace_mixed_plain_kernel(
     Lane L;
     L.active = true;
     lane_begin_ray(L, g, f, ray, btx);
-    bool done = lane_launch<STENCIL, G, IP>(L, g, f, q, gmask);
+    bool done = lane_launch<STENCIL, G, IP, FIRST>(L, g, f, q, gmask);
     // the landing state stays in registers here (a shared-memory slot per
     // thread would take L1 that the sample gathers use; measured 3 % slower on
     // the 495k-ray batch), unlike in the persistent kernel
@@ -1079,7 +1080,7 @@ __global__ void __launch_bounds__(128, G == 1 ? 3 : 2) trace_mixed_plain_kernel(
     // bounded: every attempt counts against max_steps, so max_steps + 1 attempts end every ray
     const long long max_att = (long long)f.max_steps + 2;
     for (long long it = 0; it < max_att && !done; ++it) {
-        lane_attempt<STENCIL, G, IP>(L, g, f, T, q, gmask);
+        lane_attempt<STENCIL, G, IP, FIRST>(L, g, f, T, q, gmask);
         done = lane_end_attempt(L, g, f, land);
     }
     if (!done) L.status = RT_RAY_MAX_STEPS;
@@ -1093,7 +1094,7 @@ template <int STENCIL, int G, int IP>
 __global__ void __launch_bounds__(128, G == 1 ? 3 : 2) trace_mixed_persistent_kernel(GridDev g, FanDev f,
                                                                      rt_ray_result *__restrict__ out,
                                                                      unsigned long long *__restrict__ counter) {
-    constexpr bool FIRST = G == 1 && STENCIL != RT_STENCIL_GATHER;
+    constexpr bool FIRST = G > 1 || STENCIL != RT_STENCIL_GATHER;  // see appleton_hartree
     __shared__ Tableau T;
     __shared__ Base32 btx;
     __shared__ LandState land[128];
@@ -1167,6 +1168,7 @@ __global__ void __launch_bounds__(128, 2) trace_mixed_fans_kernel(GridDev g, con
                                                                   const long long *__restrict__ first, int n_fans,
                                                                   int integrator, rt_ray_result *__restrict__ out) {
     constexpr int G = 4;
+    constexpr bool FIRST = true;  // see appleton_hartree
     __shared__ Tableau T;
     load_tableau(T, integrator);
     const long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / G;
@@ -1183,11 +1185,11 @@ __global__ void __launch_bounds__(128, 2) trace_mixed_fans_kernel(GridDev g, con
     Lane L;
     L.active = true;
     lane_begin_ray(L, g, f, claim_to_ray(f, i - first[lo]), tx_base(g, f));
-    bool done = lane_launch<STENCIL, G, IP>(L, g, f, q, gmask);
+    bool done = lane_launch<STENCIL, G, IP, FIRST>(L, g, f, q, gmask);
     LandState land;
     const long long max_att = (long long)f.max_steps + 2;
     for (long long it = 0; it < max_att && !done; ++it) {
-        lane_attempt<STENCIL, G, IP>(L, g, f, T, q, gmask);
+        lane_attempt<STENCIL, G, IP, FIRST>(L, g, f, T, q, gmask);
         done = lane_end_attempt(L, g, f, land);
     }
     if (!done) L.status = RT_RAY_MAX_STEPS;
@@ -1267,13 +1269,13 @@ __global__ void eval_rhs_kernel(GridDev g, const double *__restrict__ ys, double
     base_from_state(g, y, b);
     float d[6] = {0, 0, 0, 0, 0, 0}, dyf[6], m2;
     if (g.interp == 1) {
-        if (stencil == RT_STENCIL_TABLE) rhs_mixed<RT_STENCIL_TABLE, 1, 1>(g, rp, b, d, dyf, &m2, 0, 0u);
-        else if (stencil == RT_STENCIL_GATHER) rhs_mixed<RT_STENCIL_GATHER, 1, 1>(g, rp, b, d, dyf, &m2, 0, 0u);
-        else rhs_mixed<RT_STENCIL_QUAD, 1, 1>(g, rp, b, d, dyf, &m2, 0, 0u);
+        if (stencil == RT_STENCIL_TABLE) rhs_mixed<RT_STENCIL_TABLE, 1, 1, true>(g, rp, b, d, dyf, &m2, 0, 0u);
+        else if (stencil == RT_STENCIL_GATHER) rhs_mixed<RT_STENCIL_GATHER, 1, 1, true>(g, rp, b, d, dyf, &m2, 0, 0u);
+        else rhs_mixed<RT_STENCIL_QUAD, 1, 1, true>(g, rp, b, d, dyf, &m2, 0, 0u);
     } else {
-        if (stencil == RT_STENCIL_TABLE) rhs_mixed<RT_STENCIL_TABLE, 1, 0>(g, rp, b, d, dyf, &m2, 0, 0u);
-        else if (stencil == RT_STENCIL_GATHER) rhs_mixed<RT_STENCIL_GATHER, 1, 0>(g, rp, b, d, dyf, &m2, 0, 0u);
-        else rhs_mixed<RT_STENCIL_QUAD, 1, 0>(g, rp, b, d, dyf, &m2, 0, 0u);
+        if (stencil == RT_STENCIL_TABLE) rhs_mixed<RT_STENCIL_TABLE, 1, 0, true>(g, rp, b, d, dyf, &m2, 0, 0u);
+        else if (stencil == RT_STENCIL_GATHER) rhs_mixed<RT_STENCIL_GATHER, 1, 0, true>(g, rp, b, d, dyf, &m2, 0, 0u);
+        else rhs_mixed<RT_STENCIL_QUAD, 1, 0, true>(g, rp, b, d, dyf, &m2, 0, 0u);
     }
 #pragma unroll
     for (int c = 0; c < 6; ++c) dys[i * 6 + c] = dyf[c];
