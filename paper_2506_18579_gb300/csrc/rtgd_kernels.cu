@@ -386,9 +386,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
                                           const float d[6], float dy[6], float *mu2, int q, unsigned gmask) {
     StageIn<float> s;
     const float xa = b.ta + g.sa * d[1], xb = b.tb + g.sb * d[2], xc = b.tc + g.sc * d[0];
-    // beyond far_stage NaN, so that the adaptive step control retries with a
-    // smaller step and a fixed step ends the ray as not finite
-    s.r = fmaxf(fmaxf(fabsf(xa), fabsf(xb)), fabsf(xc)) <= g.far_stage ? b.r + d[0] : NAN;
+    s.r = b.r + d[0];
     angle_add(b.sth, b.cth, d[1], s.sth, s.cth);
     angle_add(b.sph, b.cph, d[2], s.sph, s.cph);
     s.k[0] = b.k[0] + d[3];
@@ -401,6 +399,9 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
     const bool in_b = stage_cell(b.ib, xb, g.n_lon, ib, tb);
     const bool in_c = stage_cell(b.ic, xc, g.n_alt, ic, tc);
     const bool inside = in_a & in_b & in_c;  // each axis is in bounds by itself
+    // beyond far_stage NaN, so that the adaptive step control retries with a
+    // smaller step and a fixed step ends the ray as not finite
+    const float far = fmaxf(fmaxf(fabsf(xa), fabsf(xb)), fabsf(xc)) <= g.far_stage ? 0.0f : NAN;
     float wa[4], da[4], wb[4], db[4], wc[4], dc[4], out[4], ref;
     constexpr int NA = 4 / G;
     const int a0 = q * NA;
@@ -467,7 +468,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
     out[0] += ref;
     // Ne = 0 outside the grid box (selects, so that samples gathered there,
     // whatever they hold, never reach the result)
-    s.X = inside ? rp.xfac * out[0] : 0.0f;
+    s.X = inside ? fmaf(rp.xfac, out[0], far) : far;
     s.dX[0] = inside ? rp.xfac * out[3] * g.sc : 0.0f;
     s.dX[1] = inside ? rp.xfac * out[1] * g.sa : 0.0f;
     s.dX[2] = inside ? rp.xfac * out[2] * g.sb : 0.0f;
