@@ -214,12 +214,6 @@ rt_err make_plan(const rt_grid *grid, const rt_fan_desc *fan, size_t n_rays, con
     if (c.stencil == RT_STENCIL_AUTO) c.stencil = RT_STENCIL_QUAD;
     if (c.stencil == RT_STENCIL_TABLE && !grid->table)
         return fail(RT_EINVAL, "stencil TABLE needs a grid created with RT_GRID_TABLE");
-    const int asked_stencil = c.stencil;  // the automatic lane choice goes by it
-    // The plain kernels read GATHER's samples from the quad layout, which every
-    // grid holds: the same values and records, 16 vector loads a stage instead
-    // of 64 (495,122 rays 77.4 -> 67.0 ms, C2 fan 21.5 -> 17.2 ms at one lane per
-    // ray, 12.6 -> 11.3 at four).
-    if (c.stencil == RT_STENCIL_GATHER && c.kernel == RT_KERNEL_PLAIN) c.stencil = RT_STENCIL_QUAD;
     if (c.order == RT_ORDER_CANONICAL && cfg == nullptr) c.order = RT_ORDER_ELEVATION_FASTEST;
     if (fan->precision == RT_FP64 && c.lanes_per_ray > 1)
         return fail(RT_EINVAL, "lanes_per_ray does not apply to the FP64 path");
@@ -234,7 +228,7 @@ rt_err make_plan(const rt_grid *grid, const rt_fan_desc *fan, size_t n_rays, con
         if (lanes == 0) {
             // as many lanes per ray as keep the fan within the resident lanes
             int occ = 0;
-            CUDA_TRY(persistent_occupancy(asked_stencil, 1, lp->threads, &occ));
+            CUDA_TRY(persistent_occupancy(c.stencil, 1, lp->threads, &occ));
             const long long resident = (long long)props(grid->device).sms * std::max(occ, 1) * lp->threads;
             lanes = 1;
             while (lanes < 4 && (long long)n_rays * lanes * 2 <= resident) lanes *= 2;
@@ -1064,7 +1058,6 @@ rt_err rt_plan_order(rt_plan *plan, const rt_ray_result *cost_dev, int32_t sprea
     }
     LaunchPlan ll = plan->lp;
     ll.kernel = RT_KERNEL_PLAIN;
-    if (ll.stencil == RT_STENCIL_GATHER) ll.stencil = RT_STENCIL_QUAD;  // as make_plan
     ll.lanes = 4;
     ll.blocks = 0;
     ll.smem = 0;

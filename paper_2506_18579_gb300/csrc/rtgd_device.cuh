@@ -1,7 +1,7 @@
 // rtgd_device.cuh -- device-side building blocks of the RTM-GD tracer.
 //
-// What the stage evaluation needs (weights and contraction for float and
-// double; the physics for float, the FP64 path's is tail64 in rtgd_fp64.cuh):
+// What the mixed path's stage evaluation needs (the FP64 path's, with its
+// roundings spelt out, is in rtgd_fp64.cuh):
 //   - p = 3 Galerkin-Difference weights and their derivatives (Appendix A),
 //   - the 4x4x4 tensor contraction of Eq. 13 giving Ne and its gradient,
 //   - the centred dipole field and its Jacobian in local spherical components,
@@ -58,102 +58,52 @@ struct GridDev {
 // psi_1 (in powers of t), of node j the piece psi_0, of node j+1 psi_{-1} and
 // of node j+2 psi_{-2}.  The global basis function is even, so the last two
 // are the first two mirrored: w_{j+1}(t) = w_j(1-t), w_{j+2}(t) = w_{j-1}(1-t).
-// w[a] / d[a] hold the weight of node j-1+a and its t-derivative.
-template <typename R>
-__device__ __forceinline__ void gd_weights(R t, R w[4], R d[4]) {
-    const R s = R(1) - t;
-    w[0] = t * (R(-0.5) + t * (R(11.0 / 12.0) + t * (R(-1.0 / 6.0) + t * (R(-5.0 / 12.0) + t * R(1.0 / 6.0)))));
-    w[1] = R(1) + t * t * (R(-2.25) + t * (R(0.5) + t * (R(1.25) - t * R(0.5))));
-    w[2] = R(1) + s * s * (R(-2.25) + s * (R(0.5) + s * (R(1.25) - s * R(0.5))));
-    w[3] = s * (R(-0.5) + s * (R(11.0 / 12.0) + s * (R(-1.0 / 6.0) + s * (R(-5.0 / 12.0) + s * R(1.0 / 6.0)))));
-    d[0] = R(-0.5) + t * (R(11.0 / 6.0) + t * (R(-0.5) + t * (R(-5.0 / 3.0) + t * R(5.0 / 6.0))));
-    d[1] = t * (R(-4.5) + t * (R(1.5) + t * (R(5.0) - t * R(2.5))));
-    d[2] = -(s * (R(-4.5) + s * (R(1.5) + s * (R(5.0) - s * R(2.5)))));
-    d[3] = -(R(-0.5) + s * (R(11.0 / 6.0) + s * (R(-0.5) + s * (R(-5.0 / 3.0) + s * R(5.0 / 6.0)))));
-}
-
-// The weights of nodes j-1 and j (and their t-derivatives) at local
-// coordinate s; mirrored (s = 1 - t, derivatives negated) they are the
-// weights of nodes j+2 and j+1.  interp 0: GD p = 3 (Appendix A); interp 1:
-// Catmull-Rom (Eq. 7), w_{-1} = (-s^3 + 2s^2 - s)/2, w_0 = (3s^3 - 5s^2 + 2)/2,
-// whose mirror images are w_2 and w_1.
-template <typename R>
-__device__ __forceinline__ void gd_half(R s, R &wm1, R &w0, R &dm1, R &d0, int interp = 0) {
-    if (interp == 1) {
-        wm1 = s * (R(-0.5) + s * (R(1) - s * R(0.5)));
-        w0 = R(1) + s * s * (R(-2.5) + s * R(1.5));
-        dm1 = R(-0.5) + s * (R(2) - s * R(1.5));
-        d0 = s * (R(-5) + s * R(4.5));
-        return;
-    }
-    wm1 = s * (R(-0.5) + s * (R(11.0 / 12.0) + s * (R(-1.0 / 6.0) + s * (R(-5.0 / 12.0) + s * R(1.0 / 6.0)))));
-    w0 = R(1) + s * s * (R(-2.25) + s * (R(0.5) + s * (R(1.25) - s * R(0.5))));
-    dm1 = R(-0.5) + s * (R(11.0 / 6.0) + s * (R(-0.5) + s * (R(-5.0 / 3.0) + s * R(5.0 / 6.0))));
-    d0 = s * (R(-4.5) + s * (R(1.5) + s * (R(5.0) - s * R(2.5))));
-}
-
-// gd_half with the interpolant fixed at compile time (IP = 0 GD, 1 CR).
-template <typename R, int IP>
-__device__ __forceinline__ void half_weights(R s, R &wm1, R &w0, R &dm1, R &d0) {
+// half_weights gives those of nodes j-1 and j and their derivatives at s = t;
+// at s = 1 - t, derivatives negated, they are those of nodes j+2 and j+1.  IP = 1:
+// Catmull-Rom (Eq. 7), w_{-1} = (-s^3 + 2s^2 - s)/2, w_0 = (3s^3 - 5s^2 + 2)/2.
+template <int IP>
+__device__ __forceinline__ void half_weights(float s, float &wm1, float &w0, float &dm1, float &d0) {
     if (IP == 1) {
-        wm1 = s * (R(-0.5) + s * (R(1) - s * R(0.5)));
-        w0 = R(1) + s * s * (R(-2.5) + s * R(1.5));
-        dm1 = R(-0.5) + s * (R(2) - s * R(1.5));
-        d0 = s * (R(-5) + s * R(4.5));
+        wm1 = s * (-0.5f + s * (1.0f - s * 0.5f));
+        w0 = 1.0f + s * s * (-2.5f + s * 1.5f);
+        dm1 = -0.5f + s * (2.0f - s * 1.5f);
+        d0 = s * (-5.0f + s * 4.5f);
     } else {
-        wm1 = s * (R(-0.5) + s * (R(11.0 / 12.0) + s * (R(-1.0 / 6.0) + s * (R(-5.0 / 12.0) + s * R(1.0 / 6.0)))));
-        w0 = R(1) + s * s * (R(-2.25) + s * (R(0.5) + s * (R(1.25) - s * R(0.5))));
-        dm1 = R(-0.5) + s * (R(11.0 / 6.0) + s * (R(-0.5) + s * (R(-5.0 / 3.0) + s * R(5.0 / 6.0))));
-        d0 = s * (R(-4.5) + s * (R(1.5) + s * (R(5.0) - s * R(2.5))));
+        wm1 = s * (-0.5f + s * (float(11.0 / 12.0) +
+                                s * (float(-1.0 / 6.0) + s * (float(-5.0 / 12.0) + s * float(1.0 / 6.0)))));
+        w0 = 1.0f + s * s * (-2.25f + s * (0.5f + s * (1.25f - s * 0.5f)));
+        dm1 = -0.5f + s * (float(11.0 / 6.0) + s * (-0.5f + s * (float(-5.0 / 3.0) + s * float(5.0 / 6.0))));
+        d0 = s * (-4.5f + s * (1.5f + s * (5.0f - s * 2.5f)));
     }
 }
 
 // All four weights of one axis, interpolant fixed at compile time: nodes j-1,
 // j from half_weights(t), nodes j+2, j+1 from its mirror half_weights(1 - t).
-template <typename R, int IP>
-__device__ __forceinline__ void axis_weights(R t, R w[4], R d[4]) {
-    R wp2, wp1, dp2, dp1;
-    half_weights<R, IP>(t, w[0], w[1], d[0], d[1]);
-    half_weights<R, IP>(R(1) - t, wp2, wp1, dp2, dp1);
+template <int IP>
+__device__ __forceinline__ void axis_weights(float t, float w[4], float d[4]) {
+    float wp2, wp1, dp2, dp1;
+    half_weights<IP>(t, w[0], w[1], d[0], d[1]);
+    half_weights<IP>(1.0f - t, wp2, wp1, dp2, dp1);
     w[2] = wp1;
     w[3] = wp2;
     d[2] = -dp1;
     d[3] = -dp2;
 }
 
-// All four weights of one axis (w[a], d[a] for node j-1+a), GD or CR.
-template <typename R>
-__device__ __forceinline__ void interp_weights(R t, R w[4], R d[4], int interp) {
-    if (interp == 1) {
-        R wm1, w0, dm1, d0, wp2, wp1, dp2, dp1;
-        gd_half<R>(t, wm1, w0, dm1, d0, 1);
-        gd_half<R>(R(1) - t, wp2, wp1, dp2, dp1, 1);
-        w[0] = wm1;
-        w[1] = w0;
-        w[2] = wp1;
-        w[3] = wp2;
-        d[0] = dm1;
-        d[1] = d0;
-        d[2] = -dp1;
-        d[3] = -dp2;
-        return;
-    }
-    gd_weights<R>(t, w, d);
-}
-
-// Eq. 13 contraction of one row of 4 altitude samples.  PACK (float only):
+// Eq. 13 contraction of one row of 4 altitude samples.  PACK:
 // packed FMAs on the sample pairs (u0, u1) and (u2, u3) against the weight
 // pairs, then one addition per sum -- four instructions fewer per two sums
 // and a shorter chain; the sum is formed in another order (pairs first).
-template <typename R, bool PACK = false>
-__device__ __forceinline__ void row4(R u0, R u1, R u2, R u3, const R wc[4], const R dc[4], R &v, R &dv) {
+template <bool PACK>
+__device__ __forceinline__ void row4(float u0, float u1, float u2, float u3, const float wc[4], const float dc[4],
+                                     float &v, float &dv) {
     v = u0 * wc[0] + u1 * wc[1] + u2 * wc[2] + u3 * wc[3];
     dv = u0 * dc[0] + u1 * dc[1] + u2 * dc[2] + u3 * dc[3];
 }
 
 template <>
-__device__ __forceinline__ void row4<float, true>(float u0, float u1, float u2, float u3, const float wc[4],
-                                                  const float dc[4], float &v, float &dv) {
+__device__ __forceinline__ void row4<true>(float u0, float u1, float u2, float u3, const float wc[4],
+                                           const float dc[4], float &v, float &dv) {
     const float2 a = make_float2(u0, u1), b = make_float2(u2, u3);
     const float2 p = __ffma2_rn(b, make_float2(wc[2], wc[3]), __fmul2_rn(a, make_float2(wc[0], wc[1])));
     const float2 q = __ffma2_rn(b, make_float2(dc[2], dc[3]), __fmul2_rn(a, make_float2(dc[0], dc[1])));
@@ -162,8 +112,7 @@ __device__ __forceinline__ void row4<float, true>(float u0, float u1, float u2, 
 }
 
 // Accumulates the (a, b) row into the lon/lat partial sums.
-template <typename R>
-__device__ __forceinline__ void acc_row(R v, R dv, R wb, R db, R &s, R &sb, R &sc) {
+__device__ __forceinline__ void acc_row(float v, float dv, float wb, float db, float &s, float &sb, float &sc) {
     s += v * wb;
     sb += v * db;
     sc += dv * wb;
@@ -177,20 +126,20 @@ __device__ __forceinline__ void acc_row(R v, R dv, R wb, R db, R &s, R &sb, R &s
 // float the sums do not cancel against the magnitude of Ne; the caller adds
 // REF back (after combining partial sums, when the rows are split).  PACK
 // selects the packed altitude rows (row4).
-#define RTGD_CONTRACT(R, PACK, ROW, REF, A0, NA, wa, da, wb, db, wc, dc, out)     \
+#define RTGD_CONTRACT(PACK, ROW, REF, A0, NA, wa, da, wb, db, wc, dc, out)        \
     do {                                                                          \
-        R n_ = R(0), na_ = R(0), nb_ = R(0), nc_ = R(0);                          \
+        float n_ = 0.0f, na_ = 0.0f, nb_ = 0.0f, nc_ = 0.0f;                      \
         _Pragma("unroll") for (int a_ = 0; a_ < (NA); ++a_) {                     \
-            R s_ = R(0), sb_ = R(0), sc_ = R(0);                                  \
+            float s_ = 0.0f, sb_ = 0.0f, sc_ = 0.0f;                              \
             _Pragma("unroll") for (int b_ = 0; b_ < 4; ++b_) {                    \
-                R u0_, u1_, u2_, u3_, v_, dv_;                                    \
+                float u0_, u1_, u2_, u3_, v_, dv_;                                \
                 ROW((A0) + a_, b_, u0_, u1_, u2_, u3_);                           \
                 u0_ -= (REF);                                                     \
                 u1_ -= (REF);                                                     \
                 u2_ -= (REF);                                                     \
                 u3_ -= (REF);                                                     \
-                row4<R, (PACK)>(u0_, u1_, u2_, u3_, wc, dc, v_, dv_);             \
-                acc_row<R>(v_, dv_, wb[b_], db[b_], s_, sb_, sc_);                \
+                row4<(PACK)>(u0_, u1_, u2_, u3_, wc, dc, v_, dv_);                \
+                acc_row(v_, dv_, wb[b_], db[b_], s_, sb_, sc_);                   \
             }                                                                     \
             n_ += s_ * wa[a_];                                                    \
             na_ += s_ * da[a_];                                                   \
@@ -257,43 +206,44 @@ __device__ __forceinline__ RayPhys<R> make_phys(const GridDev &g, double f_hz, i
 // FIRST: which product of S's sum is fused, T^2 or (4 L u) u.  Spelt out because
 // the compiler's choice has gone either way with the code around it, and the
 // records must not: each kernel states the form its records have.
-template <typename R, bool FIRST>
-__device__ __forceinline__ void appleton_hartree(R X, R L, R T, int mode, R &mu2, R &FX, R &FL, R &FT) {
-    const R u = R(1) - X;
-    const R S = fsqrt(FIRST ? __fmaf_rn(T, T, R(4) * L * u * u) : __fmaf_rn(R(4) * L * u, u, T * T));
+template <bool FIRST>
+__device__ __forceinline__ void appleton_hartree(float X, float L, float T, int mode, float &mu2, float &FX, float &FL,
+                                                 float &FT) {
+    const float u = 1.0f - X;
+    const float S = fsqrt(FIRST ? __fmaf_rn(T, T, 4.0f * L * u * u) : __fmaf_rn(4.0f * L * u, u, T * T));
     if (mode > 0) {
         // one reciprocal gives 1/S, 1/W and 1/(1 + g) = W/V with V = W + 2 L u
-        const R W = S + T;
-        const R V = W + R(2) * L * u;
-        const R SW = S * W;
-        const R m = recip(SW * V);
-        const R iS = W * V * m;
-        const R iW = S * V * m;
-        const R g = R(2) * L * u * iW;
-        const R opg = R(1) + g;
-        const R iopg = SW * W * m;
-        const R gX = R(2) * L * (R(4) * L * u * u * iS - W) * iW * iW;
-        const R gL = R(2) * u * iW - R(4) * L * u * u * u * iS * iW * iW;
-        const R gT = -g * iS;
-        mu2 = R(1) - X * iopg;
-        const R i2 = iopg * iopg;
+        const float W = S + T;
+        const float V = W + 2.0f * L * u;
+        const float SW = S * W;
+        const float m = recip(SW * V);
+        const float iS = W * V * m;
+        const float iW = S * V * m;
+        const float g = 2.0f * L * u * iW;
+        const float opg = 1.0f + g;
+        const float iopg = SW * W * m;
+        const float gX = 2.0f * L * (4.0f * L * u * u * iS - W) * iW * iW;
+        const float gL = 2.0f * u * iW - 4.0f * L * u * u * u * iS * iW * iW;
+        const float gT = -g * iS;
+        mu2 = 1.0f - X * iopg;
+        const float i2 = iopg * iopg;
         FX = (X * gX - opg) * i2;
         FL = X * gL * i2;
         FT = X * gT * i2;
     } else {
-        const R D = R(2) * u - T - S;
-        const R m = recip(S * D);  // 1/S and 1/D from one reciprocal
-        const R iS = D * m;
-        const R iD = S * m;
-        const R N = R(2) * X * u;
-        const R SX = R(-4) * L * u * iS;
-        const R SL = R(2) * u * u * iS;
-        const R ST = T * iS;
-        const R iD2 = iD * iD;
-        mu2 = R(1) - N * iD;
-        FX = (N * (R(-2) - SX) - (R(2) - R(4) * X) * D) * iD2;
+        const float D = 2.0f * u - T - S;
+        const float m = recip(S * D);  // 1/S and 1/D from one reciprocal
+        const float iS = D * m;
+        const float iD = S * m;
+        const float N = 2.0f * X * u;
+        const float SX = -4.0f * L * u * iS;
+        const float SL = 2.0f * u * u * iS;
+        const float ST = T * iS;
+        const float iD2 = iD * iD;
+        mu2 = 1.0f - N * iD;
+        FX = (N * (-2.0f - SX) - (2.0f - 4.0f * X) * D) * iD2;
         FL = N * (-SL) * iD2;
-        FT = N * (R(-1) - ST) * iD2;
+        FT = N * (-1.0f - ST) * iD2;
     }
 }
 
@@ -305,40 +255,38 @@ __device__ __forceinline__ void appleton_hartree(R X, R L, R T, int mode, R &mu2
 //   dY/dr = -3 Y / r,  dY/dth = A (-2 m_th, -m_r, 0),
 //   dY/dph = A (-2 sin m_ph, cos m_ph, -(sin m_r + cos m_th)),
 // so d|Y|^2/dx = 2 Y . dY/dx = (-6 |Y|^2 / r, 6 A^2 m_r m_th, 6 A^2 m_r sin m_ph).
-template <typename R>
 struct FieldTerms {
-    R Y[3];     // Y (units of the wave frequency)
-    R YY, kY;   // |Y|^2, k . Y
-    R gYY[3];   // d|Y|^2 / d(r, theta, phi)
-    R gkY[3];   // d(k . Y) / d(r, theta, phi) at fixed k
-    R ir;       // 1 / r
+    float Y[3];     // Y (units of the wave frequency)
+    float YY, kY;   // |Y|^2, k . Y
+    float gYY[3];   // d|Y|^2 / d(r, theta, phi)
+    float gkY[3];   // d(k . Y) / d(r, theta, phi) at fixed k
+    float ir;       // 1 / r
 };
 
-template <typename R>
-__device__ __forceinline__ FieldTerms<R> field_terms(const RayPhys<R> &rp, const StageIn<R> &s) {
-    FieldTerms<R> F;
-    const R kr = s.k[0], kt = s.k[1], kp = s.k[2];
-    const R mx = rp.m[0], my = rp.m[1], mz = rp.m[2];
-    const R mr = mx * s.sth * s.cph + my * s.sth * s.sph + mz * s.cth;
-    const R mt = mx * s.cth * s.cph + my * s.cth * s.sph - mz * s.sth;
-    const R mp = -mx * s.sph + my * s.cph;
+__device__ __forceinline__ FieldTerms field_terms(const RayPhys<float> &rp, const StageIn<float> &s) {
+    FieldTerms F;
+    const float kr = s.k[0], kt = s.k[1], kp = s.k[2];
+    const float mx = rp.m[0], my = rp.m[1], mz = rp.m[2];
+    const float mr = mx * s.sth * s.cph + my * s.sth * s.sph + mz * s.cth;
+    const float mt = mx * s.cth * s.cph + my * s.cth * s.sph - mz * s.sth;
+    const float mp = -mx * s.sph + my * s.cph;
     F.ir = recip(s.r);
-    const R q = rp.R_E * F.ir;
-    const R A = rp.ab0 * q * q * q;
-    F.Y[0] = R(-2) * A * mr;
+    const float q = rp.R_E * F.ir;
+    const float A = rp.ab0 * q * q * q;
+    F.Y[0] = -2.0f * A * mr;
     F.Y[1] = A * mt;
     F.Y[2] = A * mp;
-    const R A2 = A * A;
-    F.YY = A2 * (R(1) + R(3) * mr * mr);  // m is a unit vector
+    const float A2 = A * A;
+    F.YY = A2 * (1.0f + 3.0f * mr * mr);  // m is a unit vector
     F.kY = kr * F.Y[0] + kt * F.Y[1] + kp * F.Y[2];
-    const R smp = s.sth * mp;
-    const R A6mr = R(6) * A2 * mr;
-    F.gYY[0] = R(-6) * F.YY * F.ir;
+    const float smp = s.sth * mp;
+    const float A6mr = 6.0f * A2 * mr;
+    F.gYY[0] = -6.0f * F.YY * F.ir;
     F.gYY[1] = A6mr * mt;
     F.gYY[2] = A6mr * smp;
-    F.gkY[0] = R(-3) * F.kY * F.ir;
-    F.gkY[1] = A * (R(-2) * kr * mt - kt * mr);
-    F.gkY[2] = A * (R(-2) * kr * smp + kt * s.cth * mp - kp * (s.sth * mr + s.cth * mt));
+    F.gkY[0] = -3.0f * F.kY * F.ir;
+    F.gkY[1] = A * (-2.0f * kr * mt - kt * mr);
+    F.gkY[2] = A * (-2.0f * kr * smp + kt * s.cth * mp - kp * (s.sth * mr + s.cth * mt));
     return F;
 }
 
@@ -351,53 +299,53 @@ __device__ __forceinline__ FieldTerms<R> field_terms(const RayPhys<R> &rp, const
 //   dk_th/dP'  = (H_th/G - k_th dr + k_ph r cos dphi) / r,
 //   dk_ph/dP'  = (H_ph/G - k_ph sin dr - k_ph r cos dtheta) / (r sin).
 // F holds the field terms of the same stage; mu2_out receives mu^2.
-template <typename R, bool FIRST>
-__device__ __forceinline__ void ray_rhs(const RayPhys<R> &rp, const StageIn<R> &s, const FieldTerms<R> &F, R dy[6],
-                                        R *mu2_out) {
-    const R kr = s.k[0], kt = s.k[1], kp = s.k[2];
-    const R kk = kr * kr + kt * kt + kp * kp;
-    R Hr, Ht, Hp, Hk0, Hk1, Hk2, G, mu2;
+template <bool FIRST>
+__device__ __forceinline__ void ray_rhs(const RayPhys<float> &rp, const StageIn<float> &s, const FieldTerms &F,
+                                        float dy[6], float *mu2_out) {
+    const float kr = s.k[0], kt = s.k[1], kp = s.k[2];
+    const float kk = kr * kr + kt * kt + kp * kp;
+    float Hr, Ht, Hp, Hk0, Hk1, Hk2, G, mu2;
     if (rp.iso) {
         // no field: mu^2 = 1 - X, so H_x = grad(X)/2, H_k = k, G = -|k|^2 - X
-        mu2 = R(1) - s.X;
-        Hr = R(0.5) * s.dX[0];
-        Ht = R(0.5) * s.dX[1];
-        Hp = R(0.5) * s.dX[2];
+        mu2 = 1.0f - s.X;
+        Hr = 0.5f * s.dX[0];
+        Ht = 0.5f * s.dX[1];
+        Hp = 0.5f * s.dX[2];
         Hk0 = kr;
         Hk1 = kt;
         Hk2 = kp;
         G = -kk - s.X;
     } else {
-        const R ikk = recip(kk);
-        const R L = F.kY * F.kY * ikk;
-        R T = F.YY - L;
-        if (T < R(0)) T = R(0);
-        R Fm, FX, FL, FT;
-        appleton_hartree<R, FIRST>(s.X, L, T, rp.mode, Fm, FX, FL, FT);
+        const float ikk = recip(kk);
+        const float L = F.kY * F.kY * ikk;
+        float T = F.YY - L;
+        if (T < 0.0f) T = 0.0f;
+        float Fm, FX, FL, FT;
+        appleton_hartree<FIRST>(s.X, L, T, rp.mode, Fm, FX, FL, FT);
         mu2 = Fm;
         // mu^2 = F(X, L, T) with T = Y^2 - L: d/dY^2 = F_T, d/dL|_{Y^2} = F_L - F_T;
         // dL/dx at fixed k = c2 d(k . Y)/dx with c2 = 2 kY / |k|^2
-        const R FYL = FL - FT;
-        const R c2 = R(2) * F.kY * ikk;
-        const R cL = FYL * c2;
-        Hr = R(-0.5) * (FX * s.dX[0] + FT * F.gYY[0] + cL * F.gkY[0]);
-        Ht = R(-0.5) * (FX * s.dX[1] + FT * F.gYY[1] + cL * F.gkY[1]);
-        Hp = R(-0.5) * (FX * s.dX[2] + FT * F.gYY[2] + cL * F.gkY[2]);
+        const float FYL = FL - FT;
+        const float c2 = 2.0f * F.kY * ikk;
+        const float cL = FYL * c2;
+        Hr = -0.5f * (FX * s.dX[0] + FT * F.gYY[0] + cL * F.gkY[0]);
+        Ht = -0.5f * (FX * s.dX[1] + FT * F.gYY[1] + cL * F.gkY[1]);
+        Hp = -0.5f * (FX * s.dX[2] + FT * F.gYY[2] + cL * F.gkY[2]);
         // dL/dk_i = (2 kY / |k|^2) (Y_i - (kY / |k|^2) k_i)
-        const R kYn = F.kY * ikk;
-        const R hf = R(0.5) * cL;
+        const float kYn = F.kY * ikk;
+        const float hf = 0.5f * cL;
         Hk0 = kr - hf * (F.Y[0] - kYn * kr);
         Hk1 = kt - hf * (F.Y[1] - kYn * kt);
         Hk2 = kp - hf * (F.Y[2] - kYn * kp);
         // omega dH/domega: X, L and T all scale as omega^-2, |k|^2 as omega^-2
         G = -kk + s.X * FX + L * FL + T * FT;
     }
-    const R iG = recip(G);
-    const R ir = F.ir;
-    const R irs = ir * recip(s.sth);
-    const R dr = -Hk0 * iG;
-    const R dt = -Hk1 * iG * ir;
-    const R dp = -Hk2 * iG * irs;
+    const float iG = recip(G);
+    const float ir = F.ir;
+    const float irs = ir * recip(s.sth);
+    const float dr = -Hk0 * iG;
+    const float dt = -Hk1 * iG * ir;
+    const float dp = -Hk2 * iG * irs;
     dy[0] = dr;
     dy[1] = dt;
     dy[2] = dp;

@@ -172,11 +172,10 @@ __device__ __noinline__ void finish_result(double tx_th, double tx_ph, double az
 }
 
 // RKF45 error norm (<= 1 accepts) and step factor, as documented in rtgd.h.
-template <typename R>
-__device__ __forceinline__ R rkf45_err(R r, R sth, R kmag, const R e[6], R rtol, R atol) {
-    const R pos = fmax(fabs(e[0]), fmax(r * fabs(e[1]), r * sth * fabs(e[2])));
-    const R kerr = fmax(fabs(e[3]), fmax(fabs(e[4]), fabs(e[5])));
-    return fmax(fdiv(pos, atol + rtol * r), fdiv(kerr, rtol * fmax(kmag, R(1e-3))));
+__device__ __forceinline__ float rkf45_err(float r, float sth, float kmag, const float e[6], float rtol, float atol) {
+    const float pos = fmax(fabs(e[0]), fmax(r * fabs(e[1]), r * sth * fabs(e[2])));
+    const float kerr = fmax(fabs(e[3]), fmax(fabs(e[4]), fabs(e[5])));
+    return fmax(fdiv(pos, atol + rtol * r), fdiv(kerr, rtol * fmax(kmag, 1e-3f)));
 }
 
 // =============================================================== mixed path
@@ -347,11 +346,11 @@ __device__ __forceinline__ bool stage_cell(int i0, float t, int n, int &i, float
 template <int G, int IP>
 __device__ __forceinline__ void own_lat_weights(float ta, int q, float wa[4], float da[4]) {
     if (G == 1) {
-        axis_weights<float, IP>(ta, wa, da);
+        axis_weights<IP>(ta, wa, da);
     } else if (G == 2) {
         const bool hi = q != 0;  // rows 2, 3: nodes j+1, j+2
         float wm1, w0, dm1, d0;
-        half_weights<float, IP>(hi ? 1.0f - ta : ta, wm1, w0, dm1, d0);
+        half_weights<IP>(hi ? 1.0f - ta : ta, wm1, w0, dm1, d0);
         wa[0] = hi ? w0 : wm1;
         wa[1] = hi ? wm1 : w0;
         da[0] = hi ? -d0 : dm1;
@@ -359,7 +358,7 @@ __device__ __forceinline__ void own_lat_weights(float ta, int q, float wa[4], fl
     } else {
         const bool hi = q >= 2;
         float wm1, w0, dm1, d0;
-        half_weights<float, IP>(hi ? 1.0f - ta : ta, wm1, w0, dm1, d0);
+        half_weights<IP>(hi ? 1.0f - ta : ta, wm1, w0, dm1, d0);
         const bool outer = q == 0 || q == 3;  // nodes j-1, j+2
         wa[0] = outer ? wm1 : w0;
         da[0] = (outer ? dm1 : d0) * (hi ? -1.0f : 1.0f);
@@ -392,7 +391,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
     s.k[0] = b.k[0] + d[3];
     s.k[1] = b.k[1] + d[4];
     s.k[2] = b.k[2] + d[5];
-    const FieldTerms<float> F = field_terms<float>(rp, s);
+    const FieldTerms F = field_terms(rp, s);
     int ia, ib, ic;
     float ta, tb, tc;
     const bool in_a = stage_cell(b.ia, xa, g.n_lat, ia, ta);
@@ -406,8 +405,8 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
     constexpr int NA = 4 / G;
     const int a0 = q * NA;
     own_lat_weights<G, IP>(ta, q, wa, da);
-    axis_weights<float, IP>(tb, wb, db);
-    axis_weights<float, IP>(tc, wc, dc);
+    axis_weights<IP>(tb, wb, db);
+    axis_weights<IP>(tc, wc, dc);
     if (STENCIL == RT_STENCIL_QUAD) {
         // quad (pi, pj, k): 4 samples of cell k in padded row (pi, pj); node i-1 -> padded i
         const long long sj = g.q_alt, si = (long long)(g.n_lon + 2) * g.q_alt;
@@ -421,7 +420,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
         u2 = v_.z;                                        \
         u3 = v_.w;                                        \
     }
-        RTGD_CONTRACT(float, (G > 1), RTGD_ROWQ, ref, a0, NA, wa, da, wb, db, wc, dc, out);
+        RTGD_CONTRACT((G > 1), RTGD_ROWQ, ref, a0, NA, wa, da, wb, db, wc, dc, out);
 #undef RTGD_ROWQ
     } else if (STENCIL == RT_STENCIL_TABLE) {
         // one lane per ray: products in 64 bits.  Fewer instructions through
@@ -441,7 +440,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
         u2 = v_.z;                                  \
         u3 = v_.w;                                  \
     }
-        RTGD_CONTRACT(float, (G > 1), RTGD_ROWT, 0.0f, a0, NA, wa, da, wb, db, wc, dc, out);
+        RTGD_CONTRACT((G > 1), RTGD_ROWT, 0.0f, a0, NA, wa, da, wb, db, wc, dc, out);
 #undef RTGD_ROWT
     } else {
         const long long sj = g.p_alt, si = (long long)g.p_lon * g.p_alt;
@@ -455,7 +454,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
         u2 = __ldg(p_ + 2);                        \
         u3 = __ldg(p_ + 3);                        \
     }
-        RTGD_CONTRACT(float, (G > 1), RTGD_ROWG, ref, a0, NA, wa, da, wb, db, wc, dc, out);
+        RTGD_CONTRACT((G > 1), RTGD_ROWG, ref, a0, NA, wa, da, wb, db, wc, dc, out);
 #undef RTGD_ROWG
     }
     if (G > 1) {
@@ -472,7 +471,7 @@ __device__ __forceinline__ void rhs_mixed(const GridDev &g, const RayPhys<float>
     s.dX[0] = inside ? rp.xfac * out[3] * g.sc : 0.0f;
     s.dX[1] = inside ? rp.xfac * out[1] * g.sa : 0.0f;
     s.dX[2] = inside ? rp.xfac * out[2] * g.sb : 0.0f;
-    ray_rhs<float, FIRST>(rp, s, F, dy, mu2);
+    ray_rhs<FIRST>(rp, s, F, dy, mu2);
 }
 
 // Butcher tables in "shifted accumulator" form.  After stage s produced k_s,
@@ -708,10 +707,10 @@ __device__ __forceinline__ void lane_finish(Lane &L, const GridDev &g, const Fan
     out[L.out_id] = r;
 }
 
-// Final outputs of the mixed path's records, one thread per record (a
-// converged pass after the trace): record k of a fan holds the raw final
-// state lane_finish wrote; k is its canonical index, which gives the launch
-// azimuth.
+// Final outputs of the records, one thread per record (a converged pass after
+// the trace, mixed and FP64): record k of a fan holds the raw final state that
+// lane_finish or write_raw wrote; k is its canonical index, which gives the
+// launch azimuth.
 __global__ void finish_records_kernel(double R_E, FanDev f, rt_ray_result *__restrict__ out, long long n) {
     const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -952,7 +951,7 @@ __device__ bool lane_end_attempt(Lane &L, const GridDev &g, const FanDev &f, Lan
     bool accept = true;
     if (f.integrator == RT_RKF45) {
         const float kmag = fsqrt(L.b.k[0] * L.b.k[0] + L.b.k[1] * L.b.k[1] + L.b.k[2] * L.b.k[2]);
-        const float err = rkf45_err<float>(L.b.r, L.b.sth, kmag, ef, f.rtol_f, f.atol_f);
+        const float err = rkf45_err(L.b.r, L.b.sth, kmag, ef, f.rtol_f, f.atol_f);
         fac = step_factor_f(err);
         accept = err <= 1.0f;
     }
@@ -1353,9 +1352,12 @@ static cudaError_t launch_mixed_gi(const GridDev &g, const FanDev &f, rt_ray_res
                                    unsigned long long *counter, const LaunchPlan &lp, cudaStream_t st) {
     if (lp.kernel == RT_KERNEL_PERSISTENT) {
         trace_mixed_persistent_kernel<STENCIL, G, IP><<<lp.blocks, lp.threads, 0, st>>>(g, f, out, counter);
-    } else if constexpr (STENCIL == RT_STENCIL_GATHER) {
-        return cudaErrorInvalidValue;  // plain launches read the quad layout instead (make_plan)
     } else {
+        // GATHER's samples come from the quad layout, which every grid holds: the
+        // same values and records, 16 vector loads a stage instead of 64 (495,122
+        // rays 77.4 -> 67.0 ms, C2 fan 21.5 -> 17.2 ms at one lane per ray, 12.6 ->
+        // 11.3 at four).  The fused launches do the same.
+        constexpr int S = STENCIL == RT_STENCIL_GATHER ? RT_STENCIL_QUAD : STENCIL;
         const long long blocks = (f.n_rays * G + lp.threads - 1) / lp.threads;
         if (lp.started) {
             cudaLaunchConfig_t lc = {};
@@ -1369,9 +1371,9 @@ static cudaError_t launch_mixed_gi(const GridDev &g, const FanDev &f, rt_ray_res
             at[0].val.launchCompletionEvent.flags = 0;
             lc.attrs = at;
             lc.numAttrs = 1;
-            return cudaLaunchKernelEx(&lc, trace_mixed_plain_kernel<STENCIL, G, IP>, g, f, out);
+            return cudaLaunchKernelEx(&lc, trace_mixed_plain_kernel<S, G, IP>, g, f, out);
         }
-        trace_mixed_plain_kernel<STENCIL, G, IP><<<(unsigned)blocks, lp.threads, (size_t)lp.smem, st>>>(g, f, out);
+        trace_mixed_plain_kernel<S, G, IP><<<(unsigned)blocks, lp.threads, (size_t)lp.smem, st>>>(g, f, out);
     }
     return cudaGetLastError();
 }
