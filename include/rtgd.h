@@ -105,7 +105,9 @@ size_t rt_grid_device_bytes(const rt_grid *grid);
 enum { RT_MODE_O = 1u, RT_MODE_X = 2u };
 enum { RT_RK4 = 0, RT_RKF45 = 1 };
 enum {
-    RT_FP64 = 0,  /* every step of the path in double precision */
+    RT_FP64 = 0,  /* every step of the path in double precision (of the quantised step factor, a float
+                     logarithm picks the power of 2^(1/4) wherever it is not within 1e-3 of the
+                     next, a hundred times its error; double there) */
     RT_MIXED = 1  /* interpolation, Appleton-Hartree and derivatives in FP32; the ray's
                      position and its RK accumulation, the group path and the landing /
                      exit solve in FP64; the wave vector as a compensated pair of floats */

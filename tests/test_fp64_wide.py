@@ -61,3 +61,29 @@ def test_records_equal_the_lane_groups(variant):
         assert _rays_per_warp(sub.n_rays, sms) == 8
         assert rt.rt_trace(g, rt.Fan(sub, rt.RT_FP64)).reshape(-1, len(part)).tobytes() == \
             np.ascontiguousarray(res[:, part]).tobytes()
+
+
+@pytest.mark.gpu
+def test_captured_plan_and_noalloc_call():
+    """The same fan from a captured graph of a plan and through the entry point
+    that allocates nothing: the records of the plain call."""
+    import torch
+    w = wl.config2()
+    g = rt.Grid(w.grid, w.ne)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n_az = 2 * 32 * 6 * sms // (2 * 229) + 2
+    fan = rt.Fan(w.fan.replace(freq_mhz=[24.0], el_deg=np.linspace(4.0, 80.0, 229), rtol=1e-7,
+                               az_deg=np.linspace(0.0, 355.0, n_az)), rt.RT_FP64)
+    n = fan.n_rays
+    assert _rays_per_warp(n, sms) == 32
+    out, side, graph = torch.zeros((2, n * 64), dtype=torch.uint8, device="cuda"), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    plan = rt.Plan(g, fan)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        with torch.cuda.graph(graph, stream=side):
+            plan.execute(out[0].data_ptr(), n, stream=side.cuda_stream)
+    graph.replay()
+    rt.rt_trace_device_noalloc(g, fan, out[1].data_ptr(), n, stream=torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    ref = rt.rt_trace(g, fan).tobytes()
+    assert out[0].cpu().numpy().tobytes() == ref and out[1].cpu().numpy().tobytes() == ref
