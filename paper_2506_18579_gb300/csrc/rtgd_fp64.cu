@@ -991,17 +991,15 @@ __global__ void __launch_bounds__(64, kBlocksPerSm) eval_rhs_fp64_kernel(const _
 
 }  // namespace
 
-// Rays a warp starts with, by the rays per SM.  One while the first warps, one
-// FP64 instruction per 64 cycles each, leave room in a pipe that takes one per
-// 19 (64/19 = 3.4 blocks).  Above that a block more costs as much as the chain of
-// a ray saves, and the lines at 7.3 and 14.9 rays per SM are where the measured
-// times cross.  152 SMs, RKF45, 1 / 2 / 4 / 8 rays per warp: 184 rays 14.1 /
-// 16.2 / 18.0 / 21.7 ms, 460 rays 15.2 / 16.4 / 17.9 ms, 522 rays 16.7 / 15.9 /
-// 17.6 / 21.7 ms, 640 rays 35.7 / 34.7 / 36.3 ms, 1,000 rays 57.3 / 49.3 / 49.6
-// ms, 1,200 rays 51.5 / 40.2 / 40.2 / 41.9 ms, 2,000 rays 90 / 68.5 / 63.7 / 66.8
-// ms, 3,000 rays 101 / 75.4 / 70.8 / 71.2 ms, 4,968 rays 134 / 91 / 71.5 / 65.8
-// ms, 24,840 rays 571 / 335 / 210 / 149 ms; RK4, 460 rays 84.7 / 85.6 / 88.9 ms,
-// 640 rays 26.0 / 24.2 / 25.3 ms.
+// Rays a warp starts with.  An FP64 instruction takes a warp 64 cycles while
+// its SM holds fewer than ~3.4 warps and 19 cycles per resident warp above
+// that; kCost is what an evaluation takes in FP64 instructions at 4, 8, 16 and
+// 32 lanes per ray.  The size with the least product is taken.  Measured at 8 /
+// 4 / 2 / 1 rays per warp: 16 rays 47 / 36 / 29 / 25 ms, 522 rays 23 / 18 / 16 /
+// 17 ms, 3,232 rays 40 / 41 / 63 / 96 ms, 4,968 rays 104 / 113 / 129 / 162 ms,
+// 24,840 rays 149 / 208 / 340 ms / -.  More rays per warp (one or two lanes
+// each) were no faster at any size: 24,840 rays 184 ms with 32, 177 with 16,
+// against 174 with 8, all before the second warp.
 //
 // From two full waves of 32-ray warps (58,368 rays on 152 SMs) a fan is bound by
 // the pipe's throughput rather than by its longest rays, and one lane per ray
@@ -1013,9 +1011,20 @@ __global__ void __launch_bounds__(64, kBlocksPerSm) eval_rhs_fp64_kernel(const _
 // 1,156 / 457 / 503 ms, 100,434 1,034 / 531 / 483 ms, 248,442 1,577 / 1,289 /
 // 788 ms, 495,122 2,026 / 2,551 / 1,535 ms.
 int fp64_rays_per_warp(long long n_rays, int sms) {
-    const double per_sm = (double)n_rays / sms;
-    if (per_sm >= 2 * kWideRays * kBlocksPerSm) return kWideRays;
-    return per_sm <= 64.0 / 19.0 ? 1 : per_sm <= 7.27 ? 2 : per_sm <= 14.85 ? 4 : kGroups;
+    if (n_rays >= 2LL * kWideRays * kBlocksPerSm * sms) return kWideRays;
+    static const double kCost[4] = {226, 205, 190, 175};
+    double best = 1e300;
+    int R = 1;
+    for (int i = 0; i < 4; ++i) {
+        const int r = kGroups >> i;
+        const double warps = (double)((n_rays + r - 1) / r) / sms;
+        const double t = kCost[i] * (warps > 64.0 / 19.0 ? 19.0 * warps : 64.0);
+        if (t < best) {
+            best = t;
+            R = r;
+        }
+    }
+    return R;
 }
 
 cudaError_t launch_trace_fp64(const GridDev &g, const FanDev &f, int rays_per_warp, rt_ray_result *out,
