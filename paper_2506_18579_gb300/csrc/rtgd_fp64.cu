@@ -991,15 +991,18 @@ __global__ void __launch_bounds__(64, kBlocksPerSm) eval_rhs_fp64_kernel(const _
 
 }  // namespace
 
-// Rays a warp starts with.  An FP64 instruction takes a warp 64 cycles while
-// its SM holds fewer than ~3.4 warps and 19 cycles per resident warp above
-// that; kCost is what an evaluation takes in FP64 instructions at 4, 8, 16 and
-// 32 lanes per ray.  The size with the least product is taken.  Measured at 8 /
-// 4 / 2 / 1 rays per warp: 16 rays 47 / 36 / 29 / 25 ms, 522 rays 23 / 18 / 16 /
-// 17 ms, 3,232 rays 40 / 41 / 63 / 96 ms, 4,968 rays 104 / 113 / 129 / 162 ms,
-// 24,840 rays 149 / 208 / 340 ms / -.  More rays per warp (one or two lanes
-// each) were no faster at any size: 24,840 rays 184 ms with 32, 177 with 16,
-// against 174 with 8, all before the second warp.
+// Rays a warp starts with, by the rays per SM: one while a block more fits the
+// pipe beside the others (a first warp issues one FP64 instruction per 64 cycles,
+// the pipe takes one per 19: about 3.4 blocks an SM), and twice as many rays at
+// each doubling.  The first line lies a little above that: where two of the
+// longest rays are neighbours, two rays a warp lose more than they gain
+// elsewhere.  152 SMs, RKF45, a registration sector in ten ionospheres, two rays a
+// warp against one: 414 rays 1.03 to 1.11 of the time, 468 rays 0.92 to 1.01, 522
+// rays 0.92 to 1.02 (1.20 in an eleventh), 640 rays 0.77 to 0.84; four against two:
+// 800 rays 1.08, 1,000 rays 0.99, 1,220 rays 0.95.  Other fans, 1 / 2 / 4 / 8 rays
+// per warp: 2,000 rays 90 / 68.5 / 63.7 / 66.8 ms, 3,000 rays 101 / 75.4 / 70.8 /
+// 71.2 ms, 4,968 rays 134 / 91 / 71.5 / 65.8 ms, 24,840 rays 571 / 335 / 210 /
+// 149 ms.
 //
 // From two full waves of 32-ray warps (58,368 rays on 152 SMs) a fan is bound by
 // the pipe's throughput rather than by its longest rays, and one lane per ray
@@ -1011,20 +1014,9 @@ __global__ void __launch_bounds__(64, kBlocksPerSm) eval_rhs_fp64_kernel(const _
 // 1,156 / 457 / 503 ms, 100,434 1,034 / 531 / 483 ms, 248,442 1,577 / 1,289 /
 // 788 ms, 495,122 2,026 / 2,551 / 1,535 ms.
 int fp64_rays_per_warp(long long n_rays, int sms) {
-    if (n_rays >= 2LL * kWideRays * kBlocksPerSm * sms) return kWideRays;
-    static const double kCost[4] = {226, 205, 190, 175};
-    double best = 1e300;
-    int R = 1;
-    for (int i = 0; i < 4; ++i) {
-        const int r = kGroups >> i;
-        const double warps = (double)((n_rays + r - 1) / r) / sms;
-        const double t = kCost[i] * (warps > 64.0 / 19.0 ? 19.0 * warps : 64.0);
-        if (t < best) {
-            best = t;
-            R = r;
-        }
-    }
-    return R;
+    const double per_sm = (double)n_rays / sms;
+    if (per_sm >= 2 * kWideRays * kBlocksPerSm) return kWideRays;
+    return per_sm <= 3.655 ? 1 : per_sm <= 7.266 ? 2 : per_sm <= 14.845 ? 4 : kGroups;
 }
 
 cudaError_t launch_trace_fp64(const GridDev &g, const FanDev &f, int rays_per_warp, rt_ray_result *out,
