@@ -22,9 +22,10 @@
 // mates.  Ray states live in shared memory (slots), so that regrouping moves
 // no data.  The host starts a warp with as many rays as fill the GPU
 // (fp64_rays_per_warp); a fan that fills it many times over starts with 32 rays
-// a warp, one per lane (~770 instructions for 32 evaluations, the groups of
-// four lanes ~260 for eight), and goes over to groups once 16 are left, eight of
-// those at a time.  Measured with one thread per ray / lane groups / and
+// a warp, one per lane, and goes over to groups once 16 are left, eight of those
+// at a time: 20.2 FP64 warp instructions per evaluation and ray over a 63,432-ray
+// scan, step control and launch included, where eight rays a warp take 38.9 on
+// the 24,840-ray fan.  Measured with one thread per ray / lane groups / and
 // the second warp: 16 rays RK4 without a field 133 / 32 / 24.9 ms, one RKF45
 // ray 42.5 / 16.1 / 11.9 ms (one evaluation 21.2 / 8.0 / 5.9 us), 522 rays - /
 // 19.3 / 16.6 ms, 3,232 rays - / 49.0 / 38.4 ms, the 24,840-ray fan 418 / 172 /
@@ -60,8 +61,8 @@ static_assert(kSlot % 2 == 1 && cGroup % 2 == 1 && cLane % 2 == 1 && cLane >= cF
 constexpr int kGroups = 8;    // groups of a warp at most (G = 4)
 constexpr int kBlocksPerSm = 6;
 constexpr int kWideRays = 32;  // rays that a warp of the wide kernel starts with
-// One lane per ray until this few are left.  Eight of 16 at a time cost the pipe
-// what 16 lanes of their own do, and take a cluster of long rays to its end
+// One lane per ray until this few are left.  Twice eight of 16 cost the pipe
+// about what 16 lanes of their own do, and take a cluster of long rays to its end
 // sooner.  Measured at 8 / 16 / 20 / 24: 24,840 rays 148 / 152 / 160 / 162 ms,
 // 100,434 rays 564 / 483 / 490 / 493 ms, 248,442 rays 775 / 788 / 797 / 824 ms.
 constexpr int kWideLeft = 16;
